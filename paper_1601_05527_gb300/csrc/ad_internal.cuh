@@ -212,7 +212,8 @@ struct DevBuf {
 //   big    a chunk of <= kChunk neighbours of a row of degree > kBig; the
 //          chunks of one row are consecutive tasks and the last one to finish
 //          combines their partial sums (fixed order) and writes the row;
-//   medium one row of degree in (small_max, kBig];
+//   medium one row of degree in (small_max, kBig]; the sweep puts those below
+//          kWideDegree several to a warp;
 //   small  `groups` rows of degree <= small_max, one per lane group.
 // Big tasks come first, then medium rows by decreasing degree class, then
 // small rows, so that warps striding over the task list meet similar work.
@@ -222,12 +223,17 @@ struct DevBuf {
 #endif
 constexpr int kChunk = AD_CHUNK;
 constexpr int kBig = AD_CHUNK;
+// Medium rows from this degree on take a whole warp of the sweep each: 128 entries
+// are four or more full rounds of a warp's gathers, and a row's serial chain stays
+// at 32 rounds of four loads below it.
+constexpr int kWideDegree = 128;
 
 struct RowPlan {
     int small_max = 0;          // degree bound of the small class
     int groups = 0;             // lane groups per warp the plan was built for
     int64_t n_big = 0;          // big chunk tasks
     int64_t n_medium = 0;
+    int64_t n_wide = 0;         // medium rows of degree >= kWideDegree (they come first)
     int64_t n_small_rows = 0;
     int32_t *big_row = nullptr;     // [n_big]
     int32_t *big_chunk = nullptr;   // [n_big]

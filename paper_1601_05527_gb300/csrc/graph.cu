@@ -549,8 +549,19 @@ ad_status partition_by_class(ad_graph_t g, const int8_t *cls, int64_t n, int ncl
     return AD_OK;
 }
 
-// Class of a row for a plan: -1 inactive, 0 big, 1..10 medium by decreasing
-// log2 degree, 11 small.
+// Class of a row for a plan: -1 inactive, 0 big, 1..30 medium by decreasing
+// degree, four classes per power of two (the rows that share a warp of the
+// sweep then differ by less than a quarter; its slowest row sets the trip
+// count), 31 small.
+__device__ __forceinline__ int medium_class(int d) {   // 1 <= d <= 512; d >= 4: 36 - (4 log2 d) + 1
+    if (d < 4) return 30;
+    const int lg = 31 - __clz(d);
+    return 37 - (4 * lg + ((d >> (lg - 2)) & 3));
+}
+constexpr int kSmallClass = 31;
+static_assert(kBig == 512 && kWideDegree == 128, "medium_class covers degrees up to 512");
+constexpr int kFirstNarrowClass = 10;   // medium_class(d) < 10 from d = kWideDegree on
+
 __global__ void k_row_class(const int64_t *rp, const int64_t *upos, int64_t n, int small_max, int upper,
                             int8_t *cls, int64_t *nchunks) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -559,11 +570,8 @@ __global__ void k_row_class(const int64_t *rp, const int64_t *upos, int64_t n, i
         int64_t ch = 0;
         if (d <= 0) c = -1;
         else if (d > kBig) { c = 0; ch = (d + kChunk - 1) / kChunk; }
-        else if (d <= small_max) c = 11;
-        else {
-            const int lg = 63 - __clzll((unsigned long long)d);   // floor(log2 d) in [0, 9]
-            c = (int8_t)(10 - lg);
-        }
+        else if (d <= small_max) c = kSmallClass;
+        else c = (int8_t)medium_class((int)d);
         cls[i] = c;
         nchunks[i] = ch;
     }
@@ -628,8 +636,8 @@ ad_status build_row_plan(ad_graph_t g, int groups, int small_max, bool upper_onl
     }
     start[kClasses] = total;
     const int64_t n_big_rows = start[1] - start[0];
-    const int64_t n_med = start[11] - start[1];
-    const int64_t n_small = start[12] - start[11];
+    const int64_t n_med = start[kSmallClass] - start[1];
+    const int64_t n_small = start[kSmallClass + 1] - start[kSmallClass];
     // big rows -> chunk tasks
     if (n_big_rows > 0) {
         int64_t *ch = nullptr, *first = nullptr;
@@ -655,10 +663,11 @@ ad_status build_row_plan(ad_graph_t g, int groups, int small_max, bool upper_onl
     }
     if (n_small > 0) {
         AD_TRY(dalloc_t(g, n_small, &plan.small_row));
-        AD_CUDA_TRY(cudaMemcpyAsync(plan.small_row, order + start[11], n_small * sizeof(int32_t),
+        AD_CUDA_TRY(cudaMemcpyAsync(plan.small_row, order + start[kSmallClass], n_small * sizeof(int32_t),
                                     cudaMemcpyDeviceToDevice, g->stream));
     }
     plan.n_medium = n_med;
+    plan.n_wide = start[kFirstNarrowClass] - start[1];
     plan.n_small_rows = n_small;
     AD_CUDA_TRY(cudaStreamSynchronize(g->stream));
     dfree(g, cls);

@@ -82,6 +82,7 @@ static void fill_plan(SweepArgs &a, const RowPlan &p) {
     a.big_row = p.big_row; a.big_chunk = p.big_chunk; a.medium_row = p.medium_row; a.small_row = p.small_row;
     a.big_counter = p.big_counter;
     a.n_big = p.n_big; a.n_medium = p.n_medium; a.n_small_rows = p.n_small_rows;
+    a.n_wide = p.n_wide;
     a.n_tasks = p.tasks();
 }
 
@@ -120,7 +121,7 @@ ad_status sweep_step(ad_graph_t g, ad_storage storage, int32_t R, double omega, 
     fill_plan(a, *sp);
     a.x_in = x_in; a.x_out = x_out;
     a.mm_prev_min = pmin; a.mm_prev_max = pmax; a.mm_min = mn; a.mm_max = mx;
-    return dispatch_storage(g, storage, cf, true, a, 2 * 8 * (size_t)cf.stride * sizeof(float));
+    return dispatch_storage(g, storage, cf, true, a, sweep_smem(cf.stride, g->G > 1));
 }
 
 // ----------------------------------------------------------------------------
@@ -281,7 +282,7 @@ ad_status algebraic_distance(ad_graph_t g, int32_t R, int32_t k, double omega, u
     // every iterate kept: the sweeps read and write the kept buffers directly
     const bool direct = keep && keep->every == 1 && keep->ckpt.size() == (size_t)k + 1;
     if (direct) xin = keep->ckpt[0];
-    const size_t smem = 2 * 8 * (size_t)cf.stride * sizeof(float);
+    const size_t smem = sweep_smem(cf.stride, g->G > 1);
     fill_plan(a, *sp);
     for (int32_t t = 0; t < k; ++t) {
         if (direct) xout = keep->ckpt[t + 1];

@@ -28,13 +28,19 @@
 
 // Tuning parameters (compile-time; the defaults are the measured choice on GB300).
 #ifndef AD_SWEEP_UB
-#define AD_SWEEP_UB 4          // independent row loads in flight per lane
+#define AD_SWEEP_UB 8          // independent row loads in flight per lane
+#endif
+#ifndef AD_SWEEP_UBS
+#define AD_SWEEP_UBS 4         // ... of a low-degree row
 #endif
 #ifndef AD_SWEEP_MINB
-#define AD_SWEEP_MINB 6        // resident CTAs per SM requested from ptxas for the FP32 sweep
+#define AD_SWEEP_MINB 4        // resident CTAs per SM requested from ptxas for the FP32 sweep
 #endif
 #ifndef AD_SWEEP_MINB16
 #define AD_SWEEP_MINB16 5      // ... for the 16-bit storage formats
+#endif
+#ifndef AD_DIST_UB
+#define AD_DIST_UB 4           // distance: edges of one lane group in flight
 #endif
 #ifndef AD_DIST_MINB
 #define AD_DIST_MINB 4         // ... for the distance pass
@@ -75,7 +81,8 @@ struct SweepArgs {
     const int32_t *big_row, *big_chunk, *medium_row, *small_row;
     uint32_t *big_counter;
     int64_t n_big, n_medium, n_small_rows;
-    int64_t n_tasks;
+    int64_t n_wide;        // sweep: the first n_wide medium rows take a whole warp each, the others share warps
+    int64_t n_tasks;       // distance: tasks of the plan; sweep: an upper bound (the kernel counts its own)
     int32_t stride;        // elements per row
     int32_t nchunks;       // valid 16-byte chunks per row (ceil(R / V))
     int32_t R;
@@ -116,25 +123,25 @@ struct GraphCache {
 };
 
 // task index range of warp `wid` among `W` warps: [t, t_end) stepping `step`
+// (there are at most n < 2^31 tasks)
 struct TaskIter {
-    int64_t t, t_end, step;
+    uint32_t t, t_end, step;
 };
-__device__ __forceinline__ TaskIter task_iter(int64_t n_tasks, int64_t wid, int64_t W, int blocked) {
+__device__ __forceinline__ TaskIter task_iter(uint32_t n_tasks, int blocked) {
     TaskIter it;
+    const uint32_t nw = blockDim.x >> 5, warp = threadIdx.x >> 5;
     if (blocked) {
         // a contiguous range of tasks per CTA, the CTA's warps interleaved inside
         // it: a batch's lanes then meet few graphs (each change of graph flushes
-        // the lane's min/max), and the CTA's warps share neighbouring rows
-        const int nw = blockDim.x >> 5;
-        const int64_t ncta = W / nw, cta = wid / nw;
-        const int64_t per = (n_tasks + ncta - 1) / ncta;
-        it.t = cta * per + wid % nw;
-        it.t_end = min(n_tasks, cta * per + per);
+        // the min/max), and the CTA's warps share neighbouring rows
+        const uint32_t per = (n_tasks + gridDim.x - 1) / gridDim.x;
+        it.t = min(n_tasks, blockIdx.x * per) + warp;
+        it.t_end = min(n_tasks, blockIdx.x * per + per);
         it.step = nw;
     } else {
-        it.t = wid;
+        it.t = blockIdx.x * nw + warp;
         it.t_end = n_tasks;
-        it.step = W;
+        it.step = gridDim.x * nw;
     }
     return it;
 }
@@ -205,10 +212,8 @@ __device__ __forceinline__ void accumulate(float *acc, const float *f, float w) 
 // from shared memory.
 template <bool P>
 __device__ __forceinline__ uint4 ldx(const uint4 *p) { return P ? __ldcg(p) : __ldg(p); }
-template <bool P>
-__device__ __forceinline__ float4 ldac(const float *p) {
-    return P ? *reinterpret_cast<const float4 *>(p) : __ldg(reinterpret_cast<const float4 *>(p));
-}
+// scale and centre of the frame: shared memory (single graphs) or global memory (batches)
+__device__ __forceinline__ float4 ldac(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 
 template <typename T, int LPR, int CPL>
 struct Lane {
@@ -217,123 +222,157 @@ struct Lane {
     static constexpr int G = 32 / LPR;      // groups per warp
 };
 
-// Gather-accumulate rows col[p] for p in [p0, p1) with the whole warp: group
-// grp takes every G-th neighbour.  Column indices (and weights) are read 32 at
-// a time, coalesced, and broadcast with shuffles; the next 32 are loaded
-// before the current ones are used, so their latency overlaps the row loads.
-// Each lane issues up to UB independent 16-byte row loads before it consumes
-// any of them, so that enough requests are in flight to cover the L2 latency.
-// W: edge weights present; without them no weight is read or broadcast and
-// the rows are plainly added (the same sums as fmaf with weight 1).
-template <typename T, int LPR, int CPL, bool W, bool P>
-__device__ __forceinline__ void warp_gather_w(const SweepArgs &a, int64_t p0, int64_t p1, int lane, int grp,
-                                              int gl, float (&acc)[CPL * Store<T>::V]) {
-    using L = Lane<T, LPR, CPL>;
-    constexpr int V = L::V, G = L::G;
-    constexpr int U = 32 / G;                       // neighbours per group per batch of 32
-    constexpr int UBc = AD_SWEEP_UB / CPL > 0 ? AD_SWEEP_UB / CPL : 1;
-    constexpr int UB = UBc < U ? UBc : U;          // loads in flight per chunk slot
-    const uint4 *X = reinterpret_cast<const uint4 *>(a.x_in);
-    const int64_t row_q = a.stride / V;   // 16-byte chunks per row
-    int32_t cjn = 0;
-    float wjn = 0.f;
-    if (p0 + lane < p1) {
-        cjn = ld_stream(a.col + p0 + lane);
-        if (W) wjn = ld_stream(a.w + p0 + lane);
-    }
-    for (int64_t base = p0; base < p1; base += 32) {
-        const int32_t cj = cjn;
-        const float wj = wjn;
-        const int64_t pn = base + 32 + lane;
-        if (pn < p1) {
-            cjn = ld_stream(a.col + pn);
-            if (W) wjn = ld_stream(a.w + pn);
-        }
-        const int cnt = (int)(p1 - base < 32 ? p1 - base : 32);
-#pragma unroll
-        for (int u0 = 0; u0 < U; u0 += UB) {
-            if (u0 * G >= cnt) break;
-            uint4 v[UB][CPL];
-            float wt[UB];
-#pragma unroll
-            for (int u = 0; u < UB; ++u) {
-                const int src = (u0 + u) * G + grp;
-                const int32_t nb = __shfl_sync(0xffffffffu, cj, src);
-                if (W) wt[u] = __shfl_sync(0xffffffffu, wj, src);
-#pragma unroll
-                for (int c = 0; c < CPL; ++c) {
-                    const int q = gl + c * LPR;
-                    v[u][c] = (src < cnt && q < a.nchunks) ? ldx<P>(X + (int64_t)nb * row_q + q) : make_uint4(0, 0, 0, 0);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < UB; ++u)
-#pragma unroll
-                for (int c = 0; c < CPL; ++c) {
-                    float f[V];
-                    Store<T>::unpack(v[u][c], f);
-                    accumulate<V, W>(acc + c * V, f, W ? wt[u] : 1.f);
-                }
-        }
-    }
-}
+// Gather-accumulate of CSR rows by teams of lanes.  The sweep is bound by these
+// gathers (a row of 16-byte chunks per CSR entry, from L2): what counts is how many
+// are in flight and how few instructions stand between them.  Rows of 9 .. 127
+// entries share a warp, so that their epilogues run side by side and no butterfly
+// over nearly empty groups is needed; from 128 on a row fills a warp by itself.
+// Against a warp per medium row with the min/max in registers (one sweep, GB300):
+// R-MAT 20, R = 32, FP32 410 -> 303 us (FP16 349 -> 264 us), Barabasi-Albert 200K,
+// R = 10, weighted 68 -> 39 us.  The order in which the
+// entries of a row are added is fixed: entry t of a row (of a chunk of a long
+// row) belongs to residue t mod MOD, the entries of one residue are added in
+// order, and the MOD sums are added as a binary tree over adjacent residues.
+// How many lanes share that work is free: a team is MOD / RES sub-groups of
+// LPR lanes, sub-group s holding the RES residues s RES .. s RES + RES - 1 in
+// RES accumulators per lane, and a warp holds RPW teams, a row each.
+//   MOD = G, RES = 1   the whole warp on one row (chunks, rows of many entries)
+//   MOD = G, RES > 1   several rows per warp: no butterfly over idle groups, and
+//                      the epilogue of a row runs beside those of the others
+//   MOD = 1, RES = 1   one lane group per row, added one after the other
+template <int LPR, int MOD, int RES>
+struct Team {
+    static constexpr int Q = MOD / RES;         // sub-groups of a team
+    static constexpr int TL = LPR * Q;          // lanes of a team
+    static constexpr int RPW = 32 / TL;         // teams (rows) per warp
+    static constexpr int NL = LPR > 4 ? LPR : 4;   // entries per sub-group and batch
+    static constexpr int NC = NL / LPR;         // column indices a lane loads per batch
+    static constexpr int BT = NL / RES * MOD;   // entries per team and batch
+};
 
-template <typename T, int LPR, int CPL, bool P>
-__device__ __forceinline__ void warp_gather(const SweepArgs &a, int64_t p0, int64_t p1, int lane, int grp,
-                                            int gl, float (&acc)[CPL * Store<T>::V]) {
-    if (!a.w) {   // the weighted loop reads a.w: it is reached only with weights present
-        warp_gather_w<T, LPR, CPL, false, P>(a, p0, p1, lane, grp, gl, acc);
-        return;
-    }
-    warp_gather_w<T, LPR, CPL, true, P>(a, p0, p1, lane, grp, gl, acc);
-}
-
-// Gather-accumulate a short row (<= kSmallUnroll entries per round) with one
-// lane group: all of its column indices, then all row loads, then the sums.
-constexpr int kSmallUnroll = AD_SWEEP_UB;
-template <typename T, int LPR, int CPL, bool W, bool P>
-__device__ __forceinline__ void group_gather_w(const SweepArgs &a, int64_t p0, int64_t p1, int gl,
-                                               float (&acc)[CPL * Store<T>::V]) {
-    constexpr int V = Store<T>::V;
-    constexpr int UB = (kSmallUnroll / CPL) > 0 ? (kSmallUnroll / CPL) : 1;
-    const uint4 *X = reinterpret_cast<const uint4 *>(a.x_in);
-    const int64_t row_q = a.stride / V;
-    for (int64_t base = p0; base < p1; base += UB) {
-        int32_t nb[UB];
+// One batch of a team's row: its NL entries per sub-group, at most UB row loads
+// issued before any is used.  FULL: every entry of the batch exists on every
+// lane of the warp; otherwise the entries at or past `left` are left out.
+template <typename T, int LPR, int CPL, int MOD, int RES, int UB0, bool W, bool P, bool FULL>
+__device__ __forceinline__ void gather_batch(const uint4 *const (&xl)[CPL], uint32_t row_q, const int32_t *cj,
+                                             const float *wj, int sub, int left, int maxleft,
+                                             float (&acc)[RES][CPL * Store<T>::V]) {
+    using TM = Team<LPR, MOD, RES>;
+    constexpr int V = Store<T>::V, NL = TM::NL;
+    constexpr int UB1 = UB0 / CPL > 0 ? UB0 / CPL : 1;
+    constexpr int UB = UB1 < NL ? UB1 : NL;
+#pragma unroll
+    for (int l0 = 0; l0 < NL; l0 += UB) {
+        if (!FULL && (l0 / RES) * MOD >= maxleft) break;   // warp-uniform
+        uint4 v[UB][CPL];
         float wt[UB];
 #pragma unroll
         for (int u = 0; u < UB; ++u) {
-            const bool ok = base + u < p1;
-            nb[u] = ok ? ld_stream(a.col + base + u) : 0;
-            if (W) wt[u] = ok ? ld_stream(a.w + base + u) : 0.f;
+            const int l = l0 + u;
+            const int32_t nb = __shfl_sync(0xffffffffu, cj[l / LPR], l % LPR, LPR);
+            if (W) wt[u] = __shfl_sync(0xffffffffu, wj[l / LPR], l % LPR, LPR);
+            const bool ok = FULL || (l / RES) * MOD + sub * RES + l % RES < left;
+#pragma unroll
+            for (int c = 0; c < CPL; ++c)
+                v[u][c] = ok ? ldx<P>(xl[c] + (uint64_t)(uint32_t)nb * row_q) : make_uint4(0, 0, 0, 0);
         }
-        uint4 v[UB][CPL];
-#pragma unroll
-        for (int u = 0; u < UB; ++u)
-#pragma unroll
-            for (int c = 0; c < CPL; ++c) {
-                const int q = gl + c * LPR;
-                v[u][c] = (base + u < p1 && q < a.nchunks) ? ldx<P>(X + (int64_t)nb[u] * row_q + q) : make_uint4(0, 0, 0, 0);
-            }
 #pragma unroll
         for (int u = 0; u < UB; ++u)
 #pragma unroll
             for (int c = 0; c < CPL; ++c) {
                 float f[V];
                 Store<T>::unpack(v[u][c], f);
-                accumulate<V, W>(acc + c * V, f, W ? wt[u] : 1.f);
+                accumulate<V, W>(acc[(l0 + u) % RES] + c * V, f, W ? wt[u] : 1.f);
             }
     }
 }
 
-template <typename T, int LPR, int CPL, bool P>
-__device__ __forceinline__ void group_gather(const SweepArgs &a, int64_t p0, int64_t p1, int gl,
-                                             float (&acc)[CPL * Store<T>::V]) {
+// The sum of a team's row: entries p0 .. p0 + d - 1, d the same on all lanes of
+// a team (0: no row); all 32 lanes call it.  The next batch's column indices
+// (and weights) are loaded before the current batch is used.  Every lane of
+// sub-group 0 (for RES = MOD of every one) ends with the row's sum.
+template <typename T, int LPR, int CPL, int MOD, int RES, int UB, bool W, bool P>
+__device__ __forceinline__ void team_gather_w(const SweepArgs &a, int64_t p0, int d, int lane, float (&S)[CPL * Store<T>::V]) {
+    using TM = Team<LPR, MOD, RES>;
+    constexpr int V = Store<T>::V, E = CPL * V, NC = TM::NC;
+    const int gl = lane % LPR, sub = lane % TM::TL / LPR;
+    const uint32_t row_q = (uint32_t)(a.stride / V);
+    const uint4 *xl[CPL];
+#pragma unroll
+    for (int c = 0; c < CPL; ++c)   // a lane past the row's chunks reads the last one again: its sums are not used
+        xl[c] = reinterpret_cast<const uint4 *>(a.x_in) + min(gl + c * LPR, a.nchunks - 1);
+    int maxd = d, mind = d;
+    if (TM::RPW > 1) {
+        maxd = __reduce_max_sync(0xffffffffu, d);
+        mind = __reduce_min_sync(0xffffffffu, d);
+    }
+    float acc[RES][E];
+#pragma unroll
+    for (int r = 0; r < RES; ++r)
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[r][e] = 0.f;
+    int32_t cjn[NC], off[NC];
+    float wjn[NC];
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+        const int l = i * LPR + gl;
+        off[i] = (l / RES) * MOD + sub * RES + l % RES;
+        cjn[i] = 0;
+        wjn[i] = 0.f;
+        if (off[i] < d) {
+            cjn[i] = ld_stream(a.col + p0 + off[i]);
+            if (W) wjn[i] = ld_stream(a.w + p0 + off[i]);
+        }
+    }
+    for (int b = 0; b < maxd; b += TM::BT) {
+        int32_t cj[NC];
+        float wj[NC];
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+            cj[i] = cjn[i];
+            wj[i] = wjn[i];
+            const int t = b + TM::BT + off[i];
+            if (t < d) {
+                cjn[i] = ld_stream(a.col + p0 + t);
+                if (W) wjn[i] = ld_stream(a.w + p0 + t);
+            }
+        }
+        if (b + TM::BT <= mind) gather_batch<T, LPR, CPL, MOD, RES, UB, W, P, true>(xl, row_q, cj, wj, sub, 0, 0, acc);
+        else gather_batch<T, LPR, CPL, MOD, RES, UB, W, P, false>(xl, row_q, cj, wj, sub, d - b, maxd - b, acc);
+    }
+    // the tree over the residues: inside the lane, then over the sub-groups
+#pragma unroll
+    for (int o = 1; o < RES; o <<= 1)
+#pragma unroll
+        for (int r = 0; r + o < RES; r += 2 * o)
+#pragma unroll
+            for (int e = 0; e < E; ++e) acc[r][e] += acc[r + o][e];
+#pragma unroll
+    for (int e = 0; e < E; ++e) S[e] = acc[0][e];
+#pragma unroll
+    for (int o = LPR; o < TM::TL; o <<= 1)
+#pragma unroll
+        for (int e = 0; e < E; ++e) S[e] += __shfl_xor_sync(0xffffffffu, S[e], o);
+}
+
+template <typename T, int LPR, int CPL, int MOD, int RES, int UB, bool P>
+__device__ __forceinline__ void team_gather(const SweepArgs &a, int64_t p0, int d, int lane, float (&S)[CPL * Store<T>::V]) {
     if (!a.w) {   // the weighted loop reads a.w: it is reached only with weights present
-        group_gather_w<T, LPR, CPL, false, P>(a, p0, p1, gl, acc);
+        team_gather_w<T, LPR, CPL, MOD, RES, UB, false, P>(a, p0, d, lane, S);
         return;
     }
-    group_gather_w<T, LPR, CPL, true, P>(a, p0, p1, gl, acc);
+    team_gather_w<T, LPR, CPL, MOD, RES, UB, true, P>(a, p0, d, lane, S);
+}
+
+// Residues per lane of the rows that share a warp: four accumulators of one FP32
+// chunk (four rows per warp for up to eight lanes per row), two where a lane holds
+// eight values (16-bit storage, two chunks): 64 (48) registers hold no more beside
+// the loads in flight.  Measured at R-MAT 20, R = 32, FP32: 303 us with four, 323 with two.
+constexpr int kTeamRes = 4;
+template <typename T, int LPR, int CPL>
+constexpr int team_res() {
+    constexpr int G = 32 / LPR, want = Store<T>::V * CPL <= 4 ? kTeamRes : 2;
+    return G < want ? G : want;
 }
 
 // Sum over the G groups of a warp (butterfly: every group ends with the total).
@@ -357,10 +396,27 @@ __device__ __forceinline__ void load_own(const SweepArgs &a, int64_t row, int gl
     }
 }
 
-template <typename T, int LPR, int CPL, bool P = false>
+// Running minimum / maximum of a vector in shared memory, as plain floats: the
+// bit patterns of non-negative floats order like integers, those of negative
+// ones like unsigned integers reversed.
+__device__ __forceinline__ void smem_min(float *p, float f) {
+    if (__float_as_int(f) >= 0) atomicMin(reinterpret_cast<int *>(p), __float_as_int(f));
+    else atomicMax(reinterpret_cast<unsigned int *>(p), __float_as_uint(f));
+}
+__device__ __forceinline__ void smem_max(float *p, float f) {
+    if (__float_as_int(f) >= 0) atomicMax(reinterpret_cast<int *>(p), __float_as_int(f));
+    else atomicMin(reinterpret_cast<unsigned int *>(p), __float_as_uint(f));
+}
+
+// The min/max of the stored values of one graph, in shared memory: mm[0 ..
+// stride) the minima, then the maxima.  A CTA (batches: a warp) shares one copy;
+// a row that stays inside the bounds met so far -- nearly every row -- only
+// reads them (one wavefront for all rows of a warp), and no lane keeps them in
+// registers, which the gathers need.  mm NULL: straight to the global slots.
+template <typename T, int LPR, int CPL, bool P>
 __device__ __forceinline__ void row_epilogue(const SweepArgs &a, int64_t row, int gl, const uint4 (&own)[CPL],
-                                             const float (&S)[CPL * Store<T>::V], const float *acg,
-                                             float (&mn)[CPL * Store<T>::V], float (&mx)[CPL * Store<T>::V]) {
+                                             const float (&S)[CPL * Store<T>::V], const float *acg, float *mm,
+                                             uint32_t *gmin, uint32_t *gmax) {
     constexpr int V = Store<T>::V;
     uint4 *Y = reinterpret_cast<uint4 *>(a.x_out);
     const int64_t row_q = a.stride / V;
@@ -370,23 +426,42 @@ __device__ __forceinline__ void row_epilogue(const SweepArgs &a, int64_t row, in
     for (int c = 0; c < CPL; ++c) {
         const int q = gl + c * LPR;
         if (q < a.nchunks) {
-            float y[V], o[V], A[V], C[V];
+            float y[V], o[V];
             Store<T>::unpack(own[c], y);
 #pragma unroll
-            for (int e4 = 0; e4 < V / 4; ++e4) {   // scale and centre of the row's graph (the same line for every row)
-                const float4 av = ldac<P>(acg + q * V + 4 * e4);
-                const float4 cv = ldac<P>(acg + a.stride + q * V + 4 * e4);
-                A[4 * e4] = av.x; A[4 * e4 + 1] = av.y; A[4 * e4 + 2] = av.z; A[4 * e4 + 3] = av.w;
-                C[4 * e4] = cv.x; C[4 * e4 + 1] = cv.y; C[4 * e4 + 2] = cv.z; C[4 * e4 + 3] = cv.w;
-            }
+            for (int e4 = 0; e4 < V / 4; ++e4) {   // scale and centre of the row's graph
+                const float4 av = ldac(acg + q * V + 4 * e4);
+                const float4 cv = ldac(acg + a.stride + q * V + 4 * e4);
+                const float A[4] = {av.x, av.y, av.z, av.w}, C[4] = {cv.x, cv.y, cv.z, cv.w};
 #pragma unroll
-            for (int e = 0; e < V; ++e) {
-                const float z = fmaf(om1, y[e], om * (S[c * V + e] * dinv));
-                o[e] = Store<T>::round(A[e] * (z - C[e]));
-                mn[c * V + e] = fminf(mn[c * V + e], o[e]);
-                mx[c * V + e] = fmaxf(mx[c * V + e], o[e]);
+                for (int j = 0; j < 4; ++j) {
+                    const int e = 4 * e4 + j;
+                    const float z = fmaf(om1, y[e], om * (S[c * V + e] * dinv));
+                    o[e] = Store<T>::round(A[j] * (z - C[j]));
+                }
             }
             Y[row * row_q + q] = Store<T>::pack(o);
+            if (mm) {
+#pragma unroll
+                for (int e4 = 0; e4 < V / 4; ++e4) {
+                    const float4 lo = ldac(mm + q * V + 4 * e4), hi = ldac(mm + a.stride + q * V + 4 * e4);
+                    const float *oo = o + 4 * e4;
+                    if (oo[0] < lo.x || oo[1] < lo.y || oo[2] < lo.z || oo[3] < lo.w || oo[0] > hi.x || oo[1] > hi.y ||
+                        oo[2] > hi.z || oo[3] > hi.w) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            smem_min(mm + q * V + 4 * e4 + j, oo[j]);
+                            smem_max(mm + a.stride + q * V + 4 * e4 + j, oo[j]);
+                        }
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < V; ++e) {
+                    atomicMin(gmin + q * V + e, f2ord(o[e]));
+                    atomicMax(gmax + q * V + e, f2ord(o[e]));
+                }
+            }
         }
     }
 }
@@ -414,65 +489,79 @@ __device__ __forceinline__ void load_scale(const uint32_t *pmin, const uint32_t 
 
 // Scale a = 1 / (max - min) of the previous sweep's stored values (1 before the
 // first sweep, 0 for a vector with max == min) and centre c of the stored frame
-// (the previous values of the graph's anchor vertex), once per graph and sweep,
-// so that the sweep reads them from one cached line instead of holding them in
-// registers.  Block g, one thread per 16-byte chunk.
-template <typename T>
-__global__ void k_scale_center(const uint32_t *pmin, const uint32_t *pmax, const void *x_in, const int32_t *anchor,
-                               int32_t stride, float *ac) {
+// (the previous values of the graph's anchor vertex) of one graph, written to
+// A[0 .. stride) and A[stride .. 2 stride).  One thread per 16-byte chunk.
+template <typename T, bool P>
+__device__ __forceinline__ void scale_center(const uint32_t *pmin, const uint32_t *pmax, const void *x_in, int32_t anchor,
+                                             int32_t stride, float *A) {
     constexpr int V = Store<T>::V;
-    const int g = blockIdx.x;
-    float *A = ac + (size_t)g * 2 * stride, *C = A + stride;
-    const uint4 *xa = reinterpret_cast<const uint4 *>(x_in) + (int64_t)anchor[g] * (stride / V);
+    const uint4 *xa = reinterpret_cast<const uint4 *>(x_in) + (int64_t)anchor * (stride / V);
     for (int q = threadIdx.x; q < stride / V; q += blockDim.x) {
         float f[V];
-        Store<T>::unpack(xa[q], f);
+        Store<T>::unpack(ldx<P>(xa + q), f);
 #pragma unroll
         for (int e = 0; e < V; ++e) {
             const int r = q * V + e;
             float av = 1.f;
             if (pmin) {   // FP32 on purpose: FP64 division runs on a very narrow pipe on this part
-                const float lo = ord2f(pmin[(size_t)g * stride + r]), hi = ord2f(pmax[(size_t)g * stride + r]);
+                const float lo = ord2f(P ? __ldcg(pmin + r) : pmin[r]), hi = ord2f(P ? __ldcg(pmax + r) : pmax[r]);
                 av = hi > lo ? 1.f / (hi - lo) : 0.f;
             }
             A[r] = av;
-            C[r] = f[e];
+            A[stride + r] = f[e];
         }
     }
 }
 
-// ----------------------------------------------------------------------------
-// Running min/max of the values a lane stores, for the graph `cg` of the rows
-// it handled last; flushed with atomics when the lane moves to another graph.
-// ----------------------------------------------------------------------------
-template <typename T, int LPR, int CPL>
-struct LaneStats {
-    static constexpr int V = Store<T>::V, E = CPL * V;
-    float mn[E], mx[E];
-    int cg = -1;
-    const float *acg = nullptr;   // scale and centre of graph cg
+// The same for every graph of a batch (block g), which the sweep then reads from
+// one cached line per graph; a single graph's sweep computes its own in shared memory.
+template <typename T>
+__global__ void k_scale_center(const uint32_t *pmin, const uint32_t *pmax, const void *x_in, const int32_t *anchor,
+                               int32_t stride, float *ac) {
+    const size_t g = blockIdx.x;
+    scale_center<T, false>(pmin ? pmin + g * stride : nullptr, pmax ? pmax + g * stride : nullptr, x_in, anchor[g], stride,
+                           ac + g * 2 * stride);
+}
 
-    __device__ __forceinline__ void flush(const SweepArgs &a, int gl) {
-        if (cg < 0) return;
-#pragma unroll
-        for (int c = 0; c < CPL; ++c)
-#pragma unroll
-            for (int e = 0; e < V; ++e) {
-                const int r = (gl + c * LPR) * V + e;
-                if ((gl + c * LPR) < a.nchunks && mn[c * V + e] <= mx[c * V + e]) {
-                    atomicMin(a.mm_min + (size_t)cg * a.stride + r, f2ord(mn[c * V + e]));
-                    atomicMax(a.mm_max + (size_t)cg * a.stride + r, f2ord(mx[c * V + e]));
-                }
-            }
+// ----------------------------------------------------------------------------
+// The graph a warp of a batch is in: its vertex range and min/max copy, flushed
+// to the global slots when the warp moves to another graph (tasks are ordered by
+// vertex, so a warp meets few).  A row of yet another graph in the same warp (at
+// the border of two graphs) goes to the global slots directly.
+// ----------------------------------------------------------------------------
+template <typename T>
+struct WarpGraph {
+    int g = -1;
+    int32_t lo = 0, hi = 0;   // vertices of graph g
+
+    __device__ __forceinline__ void reset(const SweepArgs &a, float *mm, int lane) {
+        for (int r = lane; r < a.stride; r += 32) {
+            mm[r] = INFINITY;
+            mm[a.stride + r] = -INFINITY;
+        }
+        __syncwarp();
     }
-    // make the lane's state describe graph `g`
-    __device__ __forceinline__ void enter(const SweepArgs &a, int gl, int g, bool flush_old) {
-        if (g == cg) return;
-        if (flush_old) flush(a, gl);
-        cg = g;
-        acg = a.ac + (size_t)g * 2 * a.stride;
-#pragma unroll
-        for (int e = 0; e < E; ++e) { mn[e] = INFINITY; mx[e] = -INFINITY; }
+    __device__ __forceinline__ void flush(const SweepArgs &a, const float *mm, int lane) const {
+        __syncwarp();
+        if (g < 0) return;
+        for (int r = lane; r < a.nchunks * Store<T>::V; r += 32)
+            if (mm[r] <= mm[a.stride + r]) {
+                atomicMin(a.mm_min + (size_t)g * a.stride + r, f2ord(mm[r]));
+                atomicMax(a.mm_max + (size_t)g * a.stride + r, f2ord(mm[a.stride + r]));
+            }
+        __syncwarp();
+    }
+    // all 32 lanes; have: the lane has a row.  True: the row is in graph g.
+    __device__ __forceinline__ bool enter(const SweepArgs &a, float *mm, int lane, bool have, int32_t row) {
+        if (__any_sync(0xffffffffu, have && !(row >= lo && row < hi))) {
+            flush(a, mm, lane);
+            const int last = __reduce_max_sync(0xffffffffu, have ? row : -1);
+            g = graph_of(a.voff, a.G, last);
+            lo = (int32_t)__ldg(a.voff + g);
+            hi = (int32_t)__ldg(a.voff + g + 1);
+            reset(a, mm, lane);
+        }
+        return row >= lo && row < hi;
     }
 };
 
@@ -507,41 +596,57 @@ __device__ __forceinline__ void sum_partials(const SweepArgs &a, int64_t t0, int
     reduce_groups<LPR, E>(S);
 }
 
-// More warps per SM hide more of the gather latency even at the cost of a few
-// spilled registers: measured best at 6 CTAs (FP32) and 5 (16-bit) per SM.
+// Registers against warps, one sweep of R-MAT 20, R = 32: FP32 with eight loads in
+// flight at 3 / 4 CTAs per SM 343 / 303 us, with four at 4 / 5 CTAs 326 / 339 us;
+// FP16 with four at 3 / 4 / 5 CTAs 314 / 275 / 264 us.
 template <typename T>
 constexpr int sweep_minb() { return sizeof(T) == 4 ? AD_SWEEP_MINB : AD_SWEEP_MINB16; }
 
 // The tasks of one sweep on this CTA, then the CTA's min/max to the sweep's
-// slots.  P: inside the persistent launch (acs = the scale and centre of the
-// single graph in shared memory).
-template <typename T, int LPR, int CPL, bool P>
-__device__ __forceinline__ void sweep_tasks(const SweepArgs &a, float *sm, const float *acs) {
+// slots.  P: inside the persistent launch.  B: a batch of graphs.  acs: scale and
+// centre of a single graph in shared memory (batches read them from a.ac); mm:
+// its min/max copy, initialised (batches: one per warp).
+template <typename T, int LPR, int CPL, bool P, bool B>
+__device__ __forceinline__ void sweep_tasks(const SweepArgs &a, const float *acs, float *mm) {
     using L = Lane<T, LPR, CPL>;
-    constexpr int V = L::V, E = L::E, G = L::G;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    constexpr int V = L::V, E = L::E, G = L::G, RES = team_res<T, LPR, CPL>();
+    constexpr int UB = AD_SWEEP_UB, UBS = AD_SWEEP_UBS;
+    using TM = Team<LPR, G, RES>;
+    const int lane = threadIdx.x & 31;
     const int grp = lane / LPR, gl = lane % LPR;
 
-    LaneStats<T, LPR, CPL> ls;
-    ls.enter(a, gl, 0, false);
-    if (P) ls.acg = acs;
-    GraphCache gcache;
-    auto row_graph = [&](int64_t row) { return a.G > 1 ? gcache.of(a.voff, a.G, row) : 0; };
+    WarpGraph<T> wg;
+    if (B) {
+        mm += (threadIdx.x >> 5) * 2 * a.stride;
+        wg.reset(a, mm, lane);
+    }
+    // epilogue of the lanes with a row (writer: the lane stores a part of it)
+    auto finish = [&](int32_t row, bool have, bool writer, const uint4 (&own)[CPL], const float (&S)[E]) {
+        if (B) {
+            const bool in = wg.enter(a, mm, lane, have, row);
+            if (writer) {
+                const int g = in ? wg.g : graph_of(a.voff, a.G, row);
+                row_epilogue<T, LPR, CPL, P>(a, row, gl, own, S, a.ac + (size_t)g * 2 * a.stride, in ? mm : nullptr,
+                                             a.mm_min + (size_t)g * a.stride, a.mm_max + (size_t)g * a.stride);
+            }
+        } else if (writer) {
+            row_epilogue<T, LPR, CPL, P>(a, row, gl, own, S, acs, mm, nullptr, nullptr);
+        }
+    };
 
-    const int64_t W = (int64_t)gridDim.x * nwarps;
-    const TaskIter it = task_iter(a.n_tasks, (int64_t)blockIdx.x * nwarps + warp, W, a.blocked);
-    for (int64_t task = it.t; task < it.t_end; task += it.step) {
-        float acc[E];
-#pragma unroll
-        for (int e = 0; e < E; ++e) acc[e] = 0.f;
-        if (task < a.n_big) {
+    const uint32_t n_big = (uint32_t)a.n_big, n_wide = (uint32_t)a.n_wide;
+    const uint32_t team_tasks = ((uint32_t)a.n_medium - n_wide + TM::RPW - 1) / TM::RPW;
+    const uint32_t n_tasks = n_big + n_wide + team_tasks + ((uint32_t)a.n_small_rows + G - 1) / G;
+    const TaskIter it = task_iter(n_tasks, B ? 1 : 0);
+    for (uint32_t task = it.t; task < it.t_end; task += it.step) {
+        float S[E];
+        if (task < n_big) {
             // ---- a chunk of a high-degree row; the last chunk combines
-            const int64_t row = a.big_row[task];
+            const int32_t row = a.big_row[task];
             const int32_t c = a.big_chunk[task];
             const int64_t rb = a.rp[row], re = a.rp[row + 1];
             const int64_t p0 = rb + (int64_t)c * kChunk, p1 = min(re, p0 + kChunk);
-            warp_gather<T, LPR, CPL, P>(a, p0, p1, lane, grp, gl, acc);
-            reduce_groups<LPR, E>(acc);
+            team_gather<T, LPR, CPL, G, 1, UB, P>(a, p0, (int)(p1 - p0), lane, S);
             float *part = a.part + task * (int64_t)a.stride;
             if (grp == 0) {
 #pragma unroll
@@ -549,13 +654,16 @@ __device__ __forceinline__ void sweep_tasks(const SweepArgs &a, float *sm, const
                     const int q = gl + cc * LPR;
                     if (q < a.nchunks) {
 #pragma unroll
-                        for (int e = 0; e < V; ++e) __stcg(part + q * V + e, acc[cc * V + e]);
+                        for (int e4 = 0; e4 < V / 4; ++e4)
+                            __stcg(reinterpret_cast<float4 *>(part + q * V) + e4,
+                                   make_float4(S[cc * V + 4 * e4], S[cc * V + 4 * e4 + 1], S[cc * V + 4 * e4 + 2],
+                                               S[cc * V + 4 * e4 + 3]));
                     }
                 }
                 __threadfence();
             }
             __syncwarp();
-            const int64_t t0 = task - c;
+            const uint32_t t0 = task - c;
             const int32_t nchunk = (int32_t)((re - rb + kChunk - 1) / kChunk);
             uint32_t old = 0;
             if (lane == 0) old = atomicAdd(a.big_counter + t0, 1u);
@@ -565,93 +673,77 @@ __device__ __forceinline__ void sweep_tasks(const SweepArgs &a, float *sm, const
                 // group g sums partials g, g + G, ... (fixed order); then the groups' sums are added
                 uint4 own[CPL];
                 load_own<T, LPR, CPL, P>(a, row, gl, own);
-                float S[E];
                 sum_partials<T, LPR, CPL>(a, t0, nchunk, grp, gl, S);
-                if (grp == 0) {
-                    ls.enter(a, gl, row_graph(row), true);
-                    row_epilogue<T, LPR, CPL, P>(a, row, gl, own, S, ls.acg, ls.mn, ls.mx);
-                }
+                finish(row, true, grp == 0, own, S);
                 if (lane == 0) a.big_counter[t0] = 0u;
             }
-        } else if (task < a.n_big + a.n_medium) {
+        } else if (task < n_big + n_wide) {
             // ---- one row, whole warp
-            const int64_t row = a.medium_row[task - a.n_big];
+            const int32_t row = a.medium_row[task - n_big];
             uint4 own[CPL];
             load_own<T, LPR, CPL, P>(a, row, gl, own);
-            warp_gather<T, LPR, CPL, P>(a, a.rp[row], a.rp[row + 1], lane, grp, gl, acc);
-            reduce_groups<LPR, E>(acc);
-            if (grp == 0) {
-                ls.enter(a, gl, row_graph(row), true);
-                row_epilogue<T, LPR, CPL, P>(a, row, gl, own, acc, ls.acg, ls.mn, ls.mx);
-            }
+            const int64_t p0 = a.rp[row];
+            team_gather<T, LPR, CPL, G, 1, UB, P>(a, p0, (int)(a.rp[row + 1] - p0), lane, S);
+            finish(row, true, grp == 0, own, S);
+        } else if (task < n_big + n_wide + team_tasks) {
+            // ---- RPW rows of about the same degree, one per team
+            const uint32_t mi = n_wide + (task - n_big - n_wide) * TM::RPW + lane / TM::TL;
+            const bool have = mi < (uint32_t)a.n_medium;
+            const int32_t row = have ? a.medium_row[mi] : 0;
+            const int64_t p0 = have ? a.rp[row] : 0;
+            const int d = have ? (int)(a.rp[row + 1] - p0) : 0;
+            uint4 own[CPL];
+            load_own<T, LPR, CPL, P>(a, row, gl, own);
+            team_gather<T, LPR, CPL, G, RES, UB, P>(a, p0, d, lane, S);
+            finish(row, have, have && lane % TM::TL < LPR, own, S);
         } else {
             // ---- G low-degree rows, one per lane group
-            const int64_t si = (task - a.n_big - a.n_medium) * G + grp;
-            if (si < a.n_small_rows) {
-                const int64_t row = a.small_row[si];
-                uint4 own[CPL];
-                load_own<T, LPR, CPL, P>(a, row, gl, own);
-                group_gather<T, LPR, CPL, P>(a, a.rp[row], a.rp[row + 1], gl, acc);
-                ls.enter(a, gl, row_graph(row), true);
-                row_epilogue<T, LPR, CPL, P>(a, row, gl, own, acc, ls.acg, ls.mn, ls.mx);
-            }
+            const uint32_t si = (task - n_big - n_wide - team_tasks) * G + grp;
+            const bool have = si < (uint32_t)a.n_small_rows;
+            const int32_t row = have ? a.small_row[si] : 0;
+            const int64_t p0 = have ? a.rp[row] : 0;
+            const int d = have ? (int)(a.rp[row + 1] - p0) : 0;
+            uint4 own[CPL];
+            load_own<T, LPR, CPL, P>(a, row, gl, own);
+            team_gather<T, LPR, CPL, 1, 1, UBS, P>(a, p0, d, lane, S);
+            finish(row, have, have, own, S);
         }
     }
-
-    // ---- min/max of what this CTA stored -> atomics
-    if (a.G > 1) {
-        // lanes of a warp that share one graph are reduced first
-        const bool same = __all_sync(0xffffffffu, ls.cg == __shfl_sync(0xffffffffu, ls.cg, 0));
-        if (same) {
-#pragma unroll
-            for (int off = LPR; off < 32; off <<= 1)
-#pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    ls.mn[e] = fminf(ls.mn[e], __shfl_xor_sync(0xffffffffu, ls.mn[e], off));
-                    ls.mx[e] = fmaxf(ls.mx[e], __shfl_xor_sync(0xffffffffu, ls.mx[e], off));
-                }
-            if (grp == 0) ls.flush(a, gl);
-        } else {
-            ls.flush(a, gl);
-        }
+    if (B) {
+        wg.flush(a, mm, lane);
         return;
     }
-#pragma unroll
-    for (int off = LPR; off < 32; off <<= 1)
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            ls.mn[e] = fminf(ls.mn[e], __shfl_xor_sync(0xffffffffu, ls.mn[e], off));
-            ls.mx[e] = fmaxf(ls.mx[e], __shfl_xor_sync(0xffffffffu, ls.mx[e], off));
-        }
-    float *smn = sm, *smx = sm + nwarps * a.stride;
-    if (grp == 0) {
-#pragma unroll
-        for (int c = 0; c < CPL; ++c)
-#pragma unroll
-            for (int e = 0; e < V; ++e) {
-                const int r = (gl + c * LPR) * V + e;
-                smn[warp * a.stride + r] = ls.mn[c * V + e];
-                smx[warp * a.stride + r] = ls.mx[c * V + e];
-            }
-    }
     __syncthreads();
-    for (int r = threadIdx.x; r < a.nchunks * V; r += blockDim.x) {
-        float lo = INFINITY, hi = -INFINITY;
-        for (int wi = 0; wi < nwarps; ++wi) {
-            lo = fminf(lo, smn[wi * a.stride + r]);
-            hi = fmaxf(hi, smx[wi * a.stride + r]);
+    for (int r = threadIdx.x; r < a.nchunks * V; r += blockDim.x)
+        if (mm[r] <= mm[a.stride + r]) {
+            atomicMin(a.mm_min + r, f2ord(mm[r]));
+            atomicMax(a.mm_max + r, f2ord(mm[a.stride + r]));
         }
-        if (lo <= hi) {
-            atomicMin(a.mm_min + r, f2ord(lo));
-            atomicMax(a.mm_max + r, f2ord(hi));
-        }
+}
+
+// Shared memory of a sweep: [2][stride] scale and centre, then the min/max
+// copies, [2][stride] each (one for a single graph, one per warp for a batch).
+__host__ __device__ constexpr size_t sweep_smem(int stride, bool batch) {
+    return (size_t)(2 + 2 * (batch ? 8 : 1)) * stride * sizeof(float);
+}
+
+__device__ __forceinline__ void reset_minmax(int32_t stride, float *mm) {
+    for (int r = threadIdx.x; r < stride; r += blockDim.x) {
+        mm[r] = INFINITY;
+        mm[stride + r] = -INFINITY;
     }
 }
 
-template <typename T, int LPR, int CPL>
+template <typename T, int LPR, int CPL, bool B>
 __global__ void __launch_bounds__(256, sweep_minb<T>()) k_sweep(SweepArgs a) {
-    extern __shared__ float sm[];   // [2][warps][stride]
-    sweep_tasks<T, LPR, CPL, false>(a, sm, nullptr);
+    extern __shared__ __align__(16) float sm[];   // sweep_smem()
+    float *mm = sm + 2 * a.stride;
+    if (!B) {
+        scale_center<T, false>(a.mm_prev_min, a.mm_prev_max, a.x_in, __ldg(a.anchor), a.stride, sm);
+        reset_minmax(a.stride, mm);
+        __syncthreads();
+    }
+    sweep_tasks<T, LPR, CPL, false, B>(a, sm, mm);
 }
 
 // ----------------------------------------------------------------------------
@@ -692,8 +784,8 @@ template <typename T, int LPR, int CPL, bool P>
 __device__ __forceinline__ void edge_rows(const SweepArgs &a, int64_t row, int64_t p0, int64_t p1, int step,
                                           int first, int gl, unsigned gmask, const float (&A2)[CPL * Store<T>::V]) {
     constexpr int V = Store<T>::V, E = CPL * V;
-    // edges of one group in flight: the largest power of two <= AD_SWEEP_UB (group_sums halves it)
-    constexpr int UB = AD_SWEEP_UB >= 8 ? 8 : AD_SWEEP_UB >= 4 ? 4 : AD_SWEEP_UB >= 2 ? 2 : 1;
+    // edges of one group in flight: a power of two (group_sums halves it)
+    constexpr int UB = AD_DIST_UB;
     const uint4 *X = reinterpret_cast<const uint4 *>(a.x_in);
     const int64_t row_q = a.stride / V;
     float yi[E];
@@ -764,7 +856,7 @@ template <typename T, int LPR, int CPL, bool P>
 __device__ __forceinline__ void distance_tasks(const SweepArgs &a) {
     using L = Lane<T, LPR, CPL>;
     constexpr int V = L::V, E = L::E, G = L::G;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31;
     const int grp = lane / LPR, gl = lane % LPR;
     const unsigned gmask = LPR == 32 ? 0xffffffffu : (((1u << LPR) - 1u) << (grp * LPR));
     float A[E], A2[E];
@@ -785,8 +877,7 @@ __device__ __forceinline__ void distance_tasks(const SweepArgs &a) {
     };
     GraphCache gcache;
     auto row_graph = [&](int64_t row) { return a.G > 1 ? gcache.of(a.voff, a.G, row) : 0; };
-    const int64_t W = (int64_t)gridDim.x * nwarps;
-    const TaskIter it = task_iter(a.n_tasks, (int64_t)blockIdx.x * nwarps + warp, W, a.blocked);
+    const TaskIter it = task_iter((uint32_t)a.n_tasks, a.blocked);
     for (int64_t task = it.t; task < it.t_end; task += it.step) {
         if (task < a.n_big) {
             const int64_t row = a.big_row[task];
@@ -888,8 +979,8 @@ __device__ __forceinline__ bool grid_barrier(const RelaxArgs &r, unsigned int ph
 template <typename T, int LPR, int CPL>
 __global__ void __launch_bounds__(256, sweep_minb<T>()) k_relax(RelaxArgs r) {
     constexpr int V = Store<T>::V;
-    extern __shared__ float sm[];   // [2][warps][stride] min/max, then [2][stride] scale and centre
-    float *acs = sm + 2 * (blockDim.x >> 5) * r.s.stride;
+    extern __shared__ __align__(16) float sm[];   // sweep_smem()
+    float *mm = sm + 2 * r.s.stride;
     // x0 <- rand(-0.5, 0.5) on every row of degree > 0
     init_rows<T>(r.s.rp, r.n, r.s.stride, r.seed_lo, r.seed_hi, r.stream_id, r.s.voff, 1, static_cast<T *>(r.x0));
     if (!grid_barrier(r, 1)) return;
@@ -901,25 +992,10 @@ __global__ void __launch_bounds__(256, sweep_minb<T>()) k_relax(RelaxArgs r) {
         a.mm_prev_max = t > 0 ? r.mm_max + (size_t)(t - 1) * a.stride : nullptr;
         a.mm_min = r.mm_min + (size_t)t * a.stride;
         a.mm_max = r.mm_max + (size_t)t * a.stride;
-        // scale and centre of this sweep (what k_scale_center computes), per CTA
-        const uint4 *xa = reinterpret_cast<const uint4 *>(a.x_in) + (int64_t)__ldg(a.anchor) * (a.stride / V);
-        for (int q = threadIdx.x; q < a.stride / V; q += blockDim.x) {
-            float f[V];
-            Store<T>::unpack(__ldcg(xa + q), f);
-#pragma unroll
-            for (int e = 0; e < V; ++e) {
-                const int rr = q * V + e;
-                float av = 1.f;
-                if (a.mm_prev_min) {
-                    const float lo = ord2f(__ldcg(a.mm_prev_min + rr)), hi = ord2f(__ldcg(a.mm_prev_max + rr));
-                    av = hi > lo ? 1.f / (hi - lo) : 0.f;
-                }
-                acs[rr] = av;
-                acs[a.stride + rr] = f[e];
-            }
-        }
+        scale_center<T, true>(a.mm_prev_min, a.mm_prev_max, a.x_in, __ldg(a.anchor), a.stride, sm);
+        reset_minmax(a.stride, mm);
         __syncthreads();
-        sweep_tasks<T, LPR, CPL, true>(a, sm, acs);
+        sweep_tasks<T, LPR, CPL, true, false>(a, sm, mm);
         if (!grid_barrier(r, (unsigned int)t + 2)) return;
     }
     SweepArgs d = r.d;
@@ -937,9 +1013,13 @@ struct Config {
 
 template <typename T, int LPR, int CPL>
 ad_status launch_sweep(ad_graph_t g, const SweepArgs &a, int blocks, size_t smem) {
-    AD_LAUNCH(k_scale_center<T>, a.G, 32, 0, g->stream, a.mm_prev_min, a.mm_prev_max, a.x_in, a.anchor, a.stride,
-              a.ac);
-    AD_LAUNCH((k_sweep<T, LPR, CPL>), blocks, 256, smem, g->stream, a);
+    if (a.G > 1) {
+        AD_LAUNCH(k_scale_center<T>, a.G, 32, 0, g->stream, a.mm_prev_min, a.mm_prev_max, a.x_in, a.anchor, a.stride,
+                  a.ac);
+        AD_LAUNCH((k_sweep<T, LPR, CPL, true>), blocks, 256, smem, g->stream, a);
+    } else {
+        AD_LAUNCH((k_sweep<T, LPR, CPL, false>), blocks, 256, smem, g->stream, a);
+    }
     return AD_OK;
 }
 template <typename T, int LPR, int CPL>
@@ -948,10 +1028,12 @@ ad_status launch_distance(ad_graph_t g, const SweepArgs &a, int blocks) {
     return AD_OK;
 }
 template <typename T, int LPR, int CPL>
-int blocks_for(bool sweep, size_t smem) {
+int blocks_for(bool sweep, bool batch, size_t smem) {
     int per_sm = 0;
-    if (sweep)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<T, LPR, CPL>, 256, smem);
+    if (sweep && batch)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<T, LPR, CPL, true>, 256, smem);
+    else if (sweep)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sweep<T, LPR, CPL, false>, 256, smem);
     else
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_distance<T, LPR, CPL>, 256, 0);
     return per_sm > 0 ? per_sm : 1;
@@ -963,7 +1045,7 @@ ad_status dispatch(ad_graph_t g, const Config &cf, bool sweep, const SweepArgs &
     // persistent grid: every SM full, but no more warps than tasks
     auto run = [&](auto lpr_c, auto cpl_c) -> ad_status {
         constexpr int LPR = decltype(lpr_c)::value, CPL = decltype(cpl_c)::value;
-        int per_sm = blocks_for<T, LPR, CPL>(sweep, smem);
+        int per_sm = blocks_for<T, LPR, CPL>(sweep, a.G > 1, smem);
         if (sweep && cf.per_sm > 0 && cf.per_sm < per_sm) per_sm = cf.per_sm;
         int64_t blocks = (int64_t)per_sm * g->num_sms;
         const int64_t need = (n_tasks + 7) / 8;
@@ -995,7 +1077,7 @@ ad_status dispatch(ad_graph_t g, const Config &cf, bool sweep, const SweepArgs &
 // as many as fit or as the larger of the two plans can use.
 template <typename T, int LPR, int CPL>
 ad_status launch_relax(ad_graph_t g, const Config &cf, RelaxArgs &r) {
-    const size_t smem = (2 * 8 + 2) * (size_t)r.s.stride * sizeof(float);
+    const size_t smem = sweep_smem(r.s.stride, false);
     int per_sm = 0;
     AD_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_relax<T, LPR, CPL>, 256, smem));
     if (per_sm < 1) return fail(AD_ERR_CUDA, "the persistent relaxation kernel does not fit on an SM");
