@@ -585,7 +585,7 @@ ad_status binned_ranks(ad_graph_t g, const float *score_dev, uint64_t seed, uint
     for (int32_t q = 0; q < g->n_deg_classes; ++q) cb[q] = std::cbrt((double)g->distinct_degrees[q]);
     double *cbrt_dc = nullptr, *h = nullptr;
     float *lo = nullptr, *xs = nullptr, *rinv = nullptr;
-    uint32_t *bin = nullptr, *key = nullptr, *rk = nullptr, *desc = nullptr, *sbin = nullptr, *order = nullptr,
+    uint32_t *bin = nullptr, *key = nullptr, *rk = nullptr, *sbin = nullptr, *order = nullptr,
              *tkey = nullptr;
     int32_t *sorted = nullptr;
     int64_t *flag = nullptr, *run_of = nullptr, *run_start = nullptr, *rval = nullptr, *row_runs = nullptr;
@@ -599,7 +599,6 @@ ad_status binned_ranks(ad_graph_t g, const float *score_dev, uint64_t seed, uint
     AD_TRY(dalloc_t(g, nnz, &bin));
     AD_TRY(dalloc_t(g, nnz, &key));
     AD_TRY(dalloc_t(g, nnz, &rk));
-    AD_TRY(dalloc_t(g, nnz, &desc));
     AD_TRY(dalloc_t(g, 1, &max_bin));
     AD_TRY(copy_in(g, cbrt_dc, cb.data(), cb.size() * sizeof(double)));
     AD_CUDA_TRY(cudaMemsetAsync(max_bin, 0, sizeof(unsigned long long), g->stream));
@@ -620,7 +619,7 @@ ad_status binned_ranks(ad_graph_t g, const float *score_dev, uint64_t seed, uint
     auto release = [&]() {
         for (void *p : {(void *)cbrt_dc, (void *)lo, (void *)h, (void *)rinv, (void *)xs, (void *)bin, (void *)key,
                         (void *)tkey, (void *)rk,
-                        (void *)desc, (void *)max_bin, (void *)sbin, (void *)sorted, (void *)flag, (void *)run_of,
+                        (void *)max_bin, (void *)sbin, (void *)sorted, (void *)flag, (void *)run_of,
                         (void *)run_start, (void *)rval, (void *)row_runs, (void *)rkey, (void *)order})
             if (p) dfree(g, p);
     };
@@ -633,7 +632,7 @@ ad_status binned_ranks(ad_graph_t g, const float *score_dev, uint64_t seed, uint
     while (((unsigned long long)1 << bbits) <= mb) ++bbits;
     AD_TRY(dalloc_t(g, nnz, &tkey));
     AD_LAUNCH(k_bin_key1, big, 256, 0, g->stream, bin, key, nnz, bbits, tkey);
-    AD_TRY(row_ranks(g, tkey, rk, desc));                                  // 1. by (bin, word)
+    AD_TRY(row_ranks(g, tkey, rk));                                  // 1. by (bin, word)
     AD_TRY(dalloc_t(g, nnz, &sorted));
     AD_TRY(dalloc_t(g, nnz, &sbin));
     AD_TRY(dalloc_t(g, nnz, &flag));
@@ -667,7 +666,7 @@ ad_status binned_ranks(ad_graph_t g, const float *score_dev, uint64_t seed, uint
                   nnz, rank_dev);
     } else {
         AD_LAUNCH(k_bin_key3, big, 256, 0, g->stream, sorted, run_of, run_start, order, nnz, key);
-        AD_TRY(row_ranks(g, key, rank_dev, desc));
+        AD_TRY(row_ranks(g, key, rank_dev));
     }
     AD_CUDA_TRY(cudaStreamSynchronize(g->stream));
     release();

@@ -226,10 +226,17 @@ __global__ void k_sel_write(const float *score, int desc, const int32_t *tg, con
 // ----------------------------------------------------------------------------
 // Per-node ranks
 // ----------------------------------------------------------------------------
-__global__ void k_entry_keys(const int64_t *eid, int64_t nnz, const float *score, int desc, uint32_t *ekey) {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x)
-        ekey[p] = score_key(score[eid[p]], desc);
-}
+// The ranking key of a CSR entry: the caller's array, or the score of its edge
+// (read where the entry is ranked: a pass that wrote the keys first cost a read
+// and a write of 4 bytes per entry and a launch).
+struct KeySrc {
+    const uint32_t *ekey;    // [nnz], or
+    const int64_t *eid;      // edge of every entry and
+    const float *score;      // score of every edge
+    __device__ __forceinline__ uint32_t operator[](int64_t p) const {
+        return ekey ? ekey[p] : score_key(__ldg(score + eid[p]), 0);
+    }
+};
 
 // Ranks are written per CSR entry in both orders; k_info then gathers them per
 // edge.  Both orders come from one ascending sort of (key, position): with lt
@@ -237,12 +244,12 @@ __global__ void k_entry_keys(const int64_t *eid, int64_t nnz, const float *score
 // rank of an entry in the descending order (ties still by ascending position)
 // is (d - leq) + (r_asc - lt).
 struct RankOut {
-    uint32_t *asc, *desc;
+    uint32_t *asc, *desc;   // either may be NULL: that order is not wanted
 };
 __device__ __forceinline__ void put_ranks(const RankOut &o, int64_t p, int d, uint32_t r_asc, uint32_t lt,
                                           uint32_t leq) {
-    o.asc[p] = r_asc;
-    o.desc[p] = (uint32_t)d - leq + (r_asc - lt);
+    if (o.asc) o.asc[p] = r_asc;
+    if (o.desc) o.desc[p] = (uint32_t)d - leq + (r_asc - lt);
 }
 
 constexpr int kSortCap = 4096;      // rows up to this degree are sorted by one CTA in shared memory
@@ -251,7 +258,7 @@ constexpr int kSortCapLarge = 12288; // ... and up to this one by one CTA holdin
 // rows of degree <= GS (8 or 32): a group of GS lanes per row, one entry per
 // lane, rank = number of smaller (key, position) pairs in the row
 template <int GS>
-__global__ void k_rank_count(const int64_t *rp, const int64_t *rows, int64_t nrows, const uint32_t *ekey,
+__global__ void k_rank_count(const int64_t *rp, const int64_t *rows, int64_t nrows, KeySrc ekey,
                              RankOut out) {
     const int lane = threadIdx.x & 31, sub = lane / GS, gl = lane % GS;
     const unsigned gmask = GS == 32 ? 0xffffffffu : (((1u << GS) - 1u) << (sub * GS));
@@ -264,15 +271,15 @@ __global__ void k_rank_count(const int64_t *rp, const int64_t *rows, int64_t nro
         int d = 0;
         if (live) { i = rows[t]; p0 = rp[i]; d = (int)(rp[i + 1] - p0); }
         const uint32_t k = gl < d ? ekey[p0 + gl] : 0xffffffffu;
-        uint32_t r = 0, lt = 0, leq = 0;
+        uint32_t lt = 0, leq = 0, eqb = 0;   // smaller keys, smaller or equal keys, equal keys at earlier positions
         // d is the same on every lane of the group, so the group's shuffles stay in step
         for (int l = 0; l < d; ++l) {
             const uint32_t o = __shfl_sync(gmask, k, l, GS);
-            r += (o < k || (o == k && l < gl)) ? 1u : 0u;
             lt += o < k ? 1u : 0u;
             leq += o <= k ? 1u : 0u;
+            eqb += (o == k && l < gl) ? 1u : 0u;
         }
-        if (gl < d) put_ranks(out, p0 + gl, d, r, lt, leq);
+        if (gl < d) put_ranks(out, p0 + gl, d, lt + eqb, lt, leq);
     }
 }
 
@@ -280,7 +287,7 @@ __global__ void k_rank_count(const int64_t *rp, const int64_t *rows, int64_t nro
 // registers (bitonic network over index lane * P + j), then writes the ranks
 template <int P>
 __global__ void __launch_bounds__(256) k_rank_wsort(const int64_t *rp, const int64_t *rows, int64_t nrows,
-                                                    const uint32_t *ekey, RankOut out) {
+                                                    KeySrc ekey, RankOut out) {
     constexpr int N = 32 * P;
     const int lane = threadIdx.x & 31;
     const int64_t W = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -394,7 +401,7 @@ constexpr size_t mid_smem(int cap) { return 2 * (size_t)cap * sizeof(unsigned lo
 static_assert(mid_smem(kSortCapLarge) <= 227 * 1024, "the large CTA sort must fit one CTA's shared memory");
 
 template <int CAP>
-__global__ void __launch_bounds__(kMidThreads) k_rank_mid(const int64_t *rp, const int64_t *rows, const uint32_t *ekey,
+__global__ void __launch_bounds__(kMidThreads) k_rank_mid(const int64_t *rp, const int64_t *rows, KeySrc ekey,
                                                           RankOut out) {
     extern __shared__ unsigned long long mid_sm[];
     unsigned long long *a = mid_sm, *b = mid_sm + CAP;
@@ -500,7 +507,7 @@ __global__ void k_big_expand(const int64_t *rows, const int64_t *rp, const int64
     }
 }
 
-__global__ void k_big_keys(const int64_t *bpos, const int32_t *bseg, int64_t nb, const uint32_t *ekey,
+__global__ void k_big_keys(const int64_t *bpos, const int32_t *bseg, int64_t nb, KeySrc ekey,
                            uint64_t *keys, int64_t *vals) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nb; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t p = bpos[i];
@@ -551,15 +558,15 @@ __global__ void k_edge_pos(const int32_t *erow, const int32_t *col, const int64_
         if (col[p] > erow[p]) epos[eid[p]] = p;
 }
 
-// per edge e = (i < j): (rank at i, rank at j, degree class of i, of j) in both orders
+// per edge e = (i < j): (rank at i, rank at j, degree class of i, of j), in the orders whose ranks are given
 __global__ void k_info(const int64_t *epos, const int64_t *mirror, const int32_t *erow, const int32_t *col,
                        const int32_t *dc, int64_t m, const uint32_t *rasc, const uint32_t *rdesc, int4 *info_asc,
                        int4 *info_desc) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t p = epos[e], q = mirror[p];
         const int di = dc[erow[p]], dj = dc[col[p]];
-        info_asc[e] = make_int4((int)rasc[p], (int)rasc[q], di, dj);
-        info_desc[e] = make_int4((int)rdesc[p], (int)rdesc[q], di, dj);
+        if (rasc) info_asc[e] = make_int4((int)rasc[p], (int)rasc[q], di, dj);
+        if (rdesc) info_desc[e] = make_int4((int)rdesc[p], (int)rdesc[q], di, dj);
     }
 }
 
@@ -609,13 +616,12 @@ __device__ __forceinline__ int graph_of_edge_warp(const int64_t *goff_e, int G, 
 }
 
 constexpr int kSharedFitProblems = 8;   // problems whose histograms a block keeps in shared memory
-__global__ void k_count_cand(const int4 *info, const int64_t *list, int64_t L, const int64_t *Ld, const int64_t *goff_e,
-                             int G, const int32_t *T, int32_t ndc, int nc, unsigned long long *hist, uint8_t *cstar) {
+__global__ void k_count_cand(const int4 *info, const int64_t *list, int64_t L, const int64_t *goff_e, int G,
+                             const int32_t *T, int32_t ndc, int nc, unsigned long long *hist, uint8_t *cstar) {
     __shared__ unsigned int h[kSharedFitProblems * 32];
     const bool shared_h = G <= kSharedFitProblems;
     for (int j = threadIdx.x; j < kSharedFitProblems * 32; j += blockDim.x) h[j] = 0;
     __syncthreads();
-    if (Ld) L = *Ld;    // length of a list compacted on the device
     const int lane = threadIdx.x & 31;
     // warp-uniform trip count, so that the whole warp meets at the histogram update
     for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < L;
@@ -697,16 +703,27 @@ __device__ __forceinline__ int64_t fit_point(const FitState &s, int cc) {
     return cc < ni ? s.lo + step * (cc + 1) : s.hi;
 }
 
+// the interval shrunk to candidate `chosen` and the one before it
+__device__ __forceinline__ FitState fit_shrink(FitState s, int chosen) {
+    const int64_t nlo = chosen > 0 ? fit_point(s, chosen - 1) : s.lo;
+    const int64_t nhi = fit_point(s, chosen);
+    s.lo = nlo;
+    s.hi = nhi;
+    s.jsel = chosen;
+    return s;
+}
+
 // The chosen candidate of a problem from its histogram of first-kept
 // candidates: the first candidate whose cumulative count reaches K becomes the
 // new upper end, the one before it the new lower end (jsel = -1: converged).
-__device__ __forceinline__ FitState fit_choose(FitState s, const unsigned long long *h) {
+__device__ __forceinline__ FitState fit_choose(FitState s, const unsigned long long *h, int pass) {
     int64_t step;
     const int ni = fit_interior(s, step);
     if (s.hi - s.lo <= 1) {
         s.jsel = -1;
         return s;
     }
+    if (pass == 0) s.base = (int64_t)h[kFitCand + 1];   // kept at lo = 0
     int64_t cum = s.base;
     int chosen = ni;                    // the upper end always reaches K
     for (int cc = 0; cc <= ni; ++cc) {
@@ -714,12 +731,35 @@ __device__ __forceinline__ FitState fit_choose(FitState s, const unsigned long l
         if (cum >= s.K) { chosen = cc; break; }
     }
     for (int cc = 0; cc < chosen; ++cc) s.base += (int64_t)h[cc];
-    const int64_t nlo = chosen > 0 ? fit_point(s, chosen - 1) : s.lo;
-    const int64_t nhi = fit_point(s, chosen);
-    s.lo = nlo;
-    s.hi = nhi;
-    s.jsel = chosen;
-    return s;
+    return fit_shrink(s, chosen);
+}
+
+// Passes that need no counting.  After pass 0 the undecided edges of a problem are
+// those first kept in (lo, hi], `base` counts the ones kept at lo.  Where every
+// change of every T inside the interval falls between two neighbouring candidates
+// (one sub-interval), all undecided edges do too: the choice follows from the
+// tables.  A problem whose base reaches K already takes the first candidate
+// every time, a converged one nothing.  (Graphs whose nodes have alike degrees
+// spend most passes so, with most edges undecided: of 128 Watts-Strogatz
+// graphs' ten passes over up to 63.6M edges, 4.8 ms, seven are of this kind.)
+// Per pass and problem, kept as maxima so that 0 is the empty state:
+struct FitSpan {
+    int32_t first;   // kFitCand - (first candidate with a T above T(lo)); 0: none
+    int32_t last;    // 1 + (last candidate with a T below T(hi)); 0: none
+};
+// the candidate that a pass chooses without counting (-1: none to choose, the
+// edges are done with); kFitCand: it has to count
+__device__ __forceinline__ int fit_known(const FitState &s, const FitSpan &f, int pass) {
+    if (s.hi - s.lo <= 1) return -1;
+    if (pass == 0) return kFitCand;
+    if (s.base >= s.K) return 0;
+    return f.first > 0 && kFitCand - f.first == f.last ? f.last : kFitCand;
+}
+// whether no problem has to count (all threads of the block call it)
+__device__ __forceinline__ bool fit_all_known(const FitState *st, const FitSpan *span, int P, int pass) {
+    int count = 0;
+    for (int k = threadIdx.x; k < P; k += blockDim.x) count |= fit_known(st[k], span[k], pass) == kFitCand;
+    return !__syncthreads_or(count);
 }
 
 // One step of the search for P problems at once, between the count of pass p
@@ -731,12 +771,21 @@ __device__ __forceinline__ FitState fit_choose(FitState s, const unsigned long l
 // is constant inside and needs no pow.  With first set, the state is the
 // initial one (e in [0, 1]: T = 1 and T = d at the ends) and nothing is chosen.
 // State, tables, ends and histograms are double-buffered by pass parity.
-__global__ void k_fit_advance(int P, int first, int last, const FitState *st_old, FitState *st_new,
+// pass: the one just counted (-1: none, the state is the initial one); list
+// selectors and lengths are kept per pass: sel 0: all edges, 1 and 2: the lists.
+__global__ void __launch_bounds__(256) k_fit_advance(int P, int pass, int last, const FitState *st_old, FitState *st_new,
                               const unsigned long long *hist, unsigned long long *hist_next, const int32_t *T_cur,
                               int32_t *T_next, const int32_t *Tlo_old, const int32_t *Thi_old, int32_t *Tlo_new,
-                              int32_t *Thi_new, const int64_t *ddeg, int32_t ndc, int64_t *next_len, int *ambiguous) {
+                              int32_t *Thi_new, const int64_t *ddeg, int32_t ndc, int32_t *sel, int64_t *len,
+                              const FitSpan *span, FitSpan *span_next, int *ambiguous) {
     const int64_t gtid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (gtid == 0) *next_len = 0;
+    if (pass >= 0) {
+        const bool known = fit_all_known(st_old, span, P, pass);
+        if (gtid == 0) {   // the next pass's list: the same one, or the other, which the compaction fills
+            sel[pass + 1] = known ? sel[pass] : sel[pass] == 1 ? 2 : 1;
+            len[pass + 1] = known ? len[pass] : 0;
+        }
+    }
     for (int64_t j = gtid; j < (int64_t)P * 32; j += (int64_t)gridDim.x * blockDim.x) hist_next[j] = 0;
     const int64_t total = (int64_t)P * kFitCand * ndc;
     for (int64_t idx = gtid; idx < total; idx += (int64_t)gridDim.x * blockDim.x) {
@@ -746,11 +795,14 @@ __global__ void k_fit_advance(int P, int first, int last, const FitState *st_old
         const int64_t d = ddeg[q];
         FitState s = st_old[k];
         int32_t tl, th;
-        if (first) {
+        if (pass < 0) {
             tl = d > 0 ? 1 : 0;
             th = (int32_t)d;
         } else {
-            s = fit_choose(s, hist + (size_t)k * 32);
+            const int known = fit_known(s, span[k], pass);
+            if (known == kFitCand) s = fit_choose(s, hist + (size_t)k * 32, pass);
+            else if (known >= 0) s = fit_shrink(s, known);
+            else s.jsel = -1;
             tl = Tlo_old[(size_t)k * ndc + q];
             th = Thi_old[(size_t)k * ndc + q];
             if (s.jsel >= 0) {
@@ -784,19 +836,85 @@ __global__ void k_fit_advance(int P, int first, int last, const FitState *st_old
             t = (int32_t)c;
         }
         T_next[idx] = t;
+        if (tl != th) {   // (a look first: most threads would only repeat what is there)
+            FitSpan *sp = span_next + k;
+            if (t != tl && *(volatile int32_t *)&sp->first < kFitCand - cc) atomicMax(&sp->first, kFitCand - cc);
+            if (t != th && *(volatile int32_t *)&sp->last < cc + 1) atomicMax(&sp->last, cc + 1);
+        }
     }
+}
+
+// First candidate at which each listed edge is kept, kFitCand when at none (pass
+// 0: kFitCand + 1 when kept at e = 0 already); per-problem histograms of it, and the
+// index itself for the compaction.  Problems whose choice is known are not counted.
+__global__ void __launch_bounds__(256) k_fit_count(const int4 *info, const int64_t *list_a, const int64_t *list_b,
+                                                   const int32_t *sel, const int64_t *len, const int64_t *goff_e, int G,
+                                                   const int32_t *T, int32_t ndc, const FitState *st, const FitSpan *span,
+                                                   int pass, unsigned long long *hist, uint8_t *cstar) {
+    __shared__ unsigned int h[kSharedFitProblems * 32];
+    const bool shared_h = G <= kSharedFitProblems;
+    for (int j = threadIdx.x; j < kSharedFitProblems * 32; j += blockDim.x) h[j] = 0;
+    if (fit_all_known(st, span, G, pass)) return;
+    const int64_t L = len[pass];
+    const int which = sel[pass];
+    const int64_t *list = which == 0 ? nullptr : which == 1 ? list_a : list_b;
+    const int lane = threadIdx.x & 31;
+    // warp-uniform trip count, so that the whole warp meets at the histogram update
+    for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < L;
+         base += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t t = base + lane;
+        int key = -1, gph = 0;
+        const int64_t e = t < L ? (list ? list[t] : t) : -1;
+        if (G > 1) gph = graph_of_edge_warp(goff_e, G, e);
+        if (t < L) {
+            const int known = fit_known(st[gph], span[gph], pass);
+            if (known != kFitCand) {
+                cstar[t] = (uint8_t)known;      // (-1: dropped)
+            } else {
+                const int4 f = info[e];
+                const int32_t *Tg = T + (size_t)gph * kFitCand * ndc;
+                int l = 0, hi = kFitCand;
+                if (pass == 0 && (f.x < 1 || f.y < 1)) {
+                    l = kFitCand + 1;           // T(d, 0) = 1: the first of an end
+                } else {
+                    while (l < hi) {
+                        const int mid = (l + hi) >> 1;
+                        const int32_t *Tm = Tg + (size_t)mid * ndc;
+                        if (f.x < Tm[f.z] || f.y < Tm[f.w]) hi = mid; else l = mid + 1;
+                    }
+                }
+                cstar[t] = (uint8_t)l;
+                key = gph * 32 + l;
+            }
+        }
+        // lanes with the same (problem, bin) add once (few bins: per-lane atomics would serialise)
+        const unsigned peers = __match_any_sync(0xffffffffu, key);
+        if (key >= 0 && (peers & ((1u << lane) - 1u)) == 0) {
+            if (shared_h) atomicAdd(&h[key], (unsigned)__popc(peers));
+            else atomicAdd(hist + key, (unsigned long long)__popc(peers));
+        }
+    }
+    __syncthreads();
+    if (shared_h)
+        for (int j = threadIdx.x; j < G * 32; j += blockDim.x)
+            if (h[j]) atomicAdd(hist + j, (unsigned long long)h[j]);
 }
 
 // undecided edges of the next pass (order within the list does not matter:
 // only counts are taken).  One atomic per block and tile: a single counter
 // takes millions of survivors in the first pass.
 constexpr int kCompactItems = 4;   // elements per thread per tile
-__global__ void __launch_bounds__(256) k_fit_compact(const int64_t *list, int64_t L, const int64_t *Ld,
+__global__ void __launch_bounds__(256) k_fit_compact(int64_t *list_a, int64_t *list_b, const int32_t *sel, int64_t *len,
                                                      const uint8_t *cstar, const int64_t *goff_e, int G,
-                                                     const FitState *st, int64_t *out, int64_t *out_len) {
+                                                     const FitState *st_old, const FitSpan *span, const FitState *st,
+                                                     int pass) {
     __shared__ unsigned int wcount[8];
     __shared__ unsigned long long base_sh;
-    if (Ld) L = *Ld;
+    if (fit_all_known(st_old, span, G, pass)) return;
+    const int64_t L = len[pass];
+    const int which = sel[pass];
+    const int64_t *list = which == 0 ? nullptr : which == 1 ? list_a : list_b;
+    int64_t *out = sel[pass + 1] == 1 ? list_a : list_b, *out_len = len + pass + 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t tile = (int64_t)blockDim.x * kCompactItems;
     for (int64_t t0 = blockIdx.x * tile; t0 < L; t0 += (int64_t)gridDim.x * tile) {
@@ -1002,7 +1120,7 @@ ad_status select_whole_graph(ad_graph_t g, const float *score, double fraction, 
 // both orders (RankOut), by degree class: register counting, warp bitonic
 // sorts, a CTA radix sort in shared memory, and the device radix sort for rows
 // above the CTA sort's capacity.
-static ad_status entry_ranks(ad_graph_t g, ad_graph_s::SelCache *c, const uint32_t *ekey, RankOut out) {
+static ad_status entry_ranks(ad_graph_t g, ad_graph_s::SelCache *c, KeySrc ekey, RankOut out) {
     auto wblocks = [&](int64_t rows_, int per_warp) {
         return (int)std::max<int64_t>(1, std::min<int64_t>((rows_ + 8 * per_warp - 1) / (8 * per_warp),
                                                            (int64_t)g->num_sms * 32));
@@ -1054,17 +1172,16 @@ static ad_status entry_ranks(ad_graph_t g, ad_graph_s::SelCache *c, const uint32
 }
 
 // Rank of every CSR entry inside its row by (key, position), ascending, for
-// caller keys (rank_out[nnz], device; desc_scratch[nnz] receives the
-// descending ranks, which the ranking yields as well).
-ad_status row_ranks(ad_graph_t g, const uint32_t *ekey, uint32_t *rank_out, uint32_t *desc_scratch) {
+// caller keys (rank_out[nnz], device).
+ad_status row_ranks(ad_graph_t g, const uint32_t *ekey, uint32_t *rank_out) {
     AD_TRY(ensure_degree_classes(g));
     ad_graph_s::SelCache *c = nullptr;
     AD_TRY(sel_cache(g, &c));
     AD_TRY(rank_lists(g, c));
     RankOut out;
     out.asc = rank_out;
-    out.desc = desc_scratch;
-    return entry_ranks(g, c, ekey, out);
+    out.desc = nullptr;
+    return entry_ranks(g, c, KeySrc{ekey, nullptr, nullptr}, out);
 }
 
 // The rows of degree above 512, by increasing id (device array, owned by the
@@ -1100,14 +1217,15 @@ static ad_status per_node_info(ad_graph_t g, const float *score, ad_mode mode, i
         if (nnz > 0)
             AD_LAUNCH(k_edge_pos, g->num_sms * 16, 256, 0, g->stream, g->erow, g->col, g->eid, nnz, c->epos);
     }
+    // both orders for the handle's own distances (a call in the other mode may follow),
+    // the one asked for on a caller's scores
+    const bool asc = own || mode != AD_MODE_GLOBAL, desc = own || mode == AD_MODE_GLOBAL;
     AD_TRY(ensure(g, c->rank2, 2 * sizeof(uint32_t) * (nnz + 1)));
+    uint32_t *ranks = static_cast<uint32_t *>(c->rank2.ptr);
     RankOut out;
-    out.asc = static_cast<uint32_t *>(c->rank2.ptr);
-    out.desc = out.asc + (nnz + 1);
-    AD_TRY(ensure(g, c->ekey, sizeof(uint32_t) * (nnz + 1)));
-    uint32_t *ekey = static_cast<uint32_t *>(c->ekey.ptr);
-    if (nnz > 0) AD_LAUNCH(k_entry_keys, g->num_sms * 16, 256, 0, g->stream, g->eid, nnz, score, 0, ekey);
-    AD_TRY(entry_ranks(g, c, ekey, out));
+    out.asc = asc ? ranks : nullptr;
+    out.desc = desc ? ranks + (nnz + 1) : nullptr;
+    AD_TRY(entry_ranks(g, c, KeySrc{nullptr, g->eid, score}, out));
     if (g->m > 0)
         AD_LAUNCH(k_info, g->num_sms * 16, 256, 0, g->stream, c->epos, g->mirror, g->erow, g->col, g->deg_class, g->m,
                   out.asc, out.desc, info_asc, info_desc);
@@ -1216,7 +1334,7 @@ static ad_status select_per_node_fit_host(ad_graph_t g, const int4 *info, double
         AD_TRY(copy_in(g, T, Th.data(), Th.size() * sizeof(int32_t)));
         AD_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * G * 32, g->stream));
         const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((L + 255) / 256, (int64_t)g->num_sms * 16));
-        AD_LAUNCH(k_count_cand, blocks, 256, 0, g->stream, info, list, L, (const int64_t *)nullptr, g->goff_e, G, T, ndc,
+        AD_LAUNCH(k_count_cand, blocks, 256, 0, g->stream, info, list, L, g->goff_e, G, T, ndc,
                   ncand, hist, cstar);
         AD_TRY(copy_out(g, hh.data(), hist, sizeof(unsigned long long) * hh.size()));
         for (int32_t k = 0; k < G; ++k) {
@@ -1295,11 +1413,11 @@ ad_status select_per_node_fit_ranked(ad_graph_t g, const uint32_t *rank, double 
         if (g->nnz > 0)
             AD_LAUNCH(k_edge_pos, g->num_sms * 16, 256, 0, g->stream, g->erow, g->col, g->eid, g->nnz, c->epos);
     }
-    AD_TRY(ensure(g, c->info_other, 2 * sizeof(int4) * (g->m + 1)));
+    AD_TRY(ensure(g, c->info_other, sizeof(int4) * (g->m + 1)));
     int4 *info = static_cast<int4 *>(c->info_other.ptr);
-    if (g->m > 0)   // the second output (the other order) is not needed: it goes to the spare half
+    if (g->m > 0)
         AD_LAUNCH(k_info, g->num_sms * 16, 256, 0, g->stream, c->epos, g->mirror, g->erow, g->col, g->deg_class, g->m,
-                  rank, rank, info, info + (g->m + 1));
+                  rank, (const uint32_t *)nullptr, info, (int4 *)nullptr);
     return fit_search(g, info, fraction, keep, n_kept, e_used);
 }
 
@@ -1326,9 +1444,9 @@ ad_status select_local_degree(ad_graph_t g, double fraction, uint8_t *keep, int6
     uint32_t *ekey = static_cast<uint32_t *>(c->ekey.ptr);
     RankOut out;
     out.asc = static_cast<uint32_t *>(c->rank2.ptr);
-    out.desc = out.asc + (nnz + 1);
+    out.desc = nullptr;
     if (nnz > 0) AD_LAUNCH(k_ld_keys, g->num_sms * 16, 256, 0, g->stream, g->rp, g->col, nnz, ekey);
-    AD_TRY(entry_ranks(g, c, ekey, out));
+    AD_TRY(entry_ranks(g, c, KeySrc{ekey, nullptr, nullptr}, out));
     return select_per_node_fit_ranked(g, out.asc, fraction, keep, n_kept, e_used);
 }
 
@@ -1368,13 +1486,16 @@ static ad_status fit_multi(ad_graph_t g, const int4 *info, int nsets, double fra
     AD_TRY(ensure(g, c->cstar, (size_t)(L0 + 1)));
     AD_TRY(ensure(g, c->list_a, sizeof(int64_t) * (L0 + 1)));
     AD_TRY(ensure(g, c->list_b, sizeof(int64_t) * (L0 + 1)));
-    AD_TRY(ensure(g, c->fit, 3 * sizeof(FitState) * P + 4 * sizeof(int64_t) + sizeof(int64_t) * (P + 1)));
+    AD_TRY(ensure(g, c->fit, 3 * sizeof(FitState) * P + (kFitPasses + 2) * sizeof(int64_t) + sizeof(int64_t) * (P + 1) +
+                                 (kFitPasses + 1) * (sizeof(FitSpan) * P + sizeof(int32_t)) + sizeof(int32_t)));
     AD_TRY(ensure(g, c->fit_tb, 4 * bsz * sizeof(int32_t)));
     FitState *stb = static_cast<FitState *>(c->fit.ptr);          // [0], [1]: by pass parity; [2]: initial
     FitState *st[2] = {stb, stb + P};
-    int64_t *len = reinterpret_cast<int64_t *>(stb + 3 * P);      // [0], [1]: list lengths; [2]: ambiguity flag
-    int *amb = reinterpret_cast<int *>(len + 2);
-    int64_t *goff = len + 4;
+    int64_t *goff = reinterpret_cast<int64_t *>(stb + 3 * P);
+    int64_t *len = goff + P + 1;                                  // list length of each pass
+    FitSpan *span = reinterpret_cast<FitSpan *>(len + kFitPasses + 2);   // [pass][P]
+    int32_t *sel = reinterpret_cast<int32_t *>(span + (size_t)(kFitPasses + 1) * P);   // list of each pass
+    int *amb = sel + kFitPasses + 1;
     int32_t *tb = static_cast<int32_t *>(c->fit_tb.ptr);
     int32_t *Tlo[2] = {tb, tb + bsz}, *Thi[2] = {tb + 2 * bsz, tb + 3 * bsz};
     int32_t *T[2] = {static_cast<int32_t *>(c->T.ptr), static_cast<int32_t *>(c->T.ptr) + tsz};
@@ -1385,23 +1506,26 @@ static ad_status fit_multi(ad_graph_t g, const int4 *info, int nsets, double fra
     const int64_t *ddeg = static_cast<const int64_t *>(c->ddeg.ptr);
     AD_TRY(copy_in(g, stb + 2 * P, sh.data(), sizeof(FitState) * P));
     AD_TRY(copy_in(g, goff, pgoff.data(), sizeof(int64_t) * (P + 1)));
-    AD_CUDA_TRY(cudaMemsetAsync(len, 0, 4 * sizeof(int64_t), g->stream));
+    AD_CUDA_TRY(cudaMemsetAsync(span, 0, (kFitPasses + 1) * (sizeof(FitSpan) * P + sizeof(int32_t)) + sizeof(int32_t),
+                                g->stream));
+    AD_TRY(copy_in(g, len, &L0, sizeof(int64_t)));
     const int big = g->num_sms * 16;
     const int ablocks = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)tsz + 255) / 256, big));
     const int cblocks = (int)std::max<int64_t>(1, std::min<int64_t>((L0 + 255) / 256, big));
     // initial state, ends and the tables of pass 0
-    AD_LAUNCH(k_fit_advance, ablocks, 256, 0, g->stream, P, 1, 0, stb + 2 * P, st[0], hist[1], hist[0], T[1], T[0],
-              Tlo[1], Thi[1], Tlo[0], Thi[0], ddeg, ndc, len + 1, amb);
+    AD_LAUNCH(k_fit_advance, ablocks, 256, 0, g->stream, P, -1, 0, stb + 2 * P, st[0], hist[1], hist[0], T[1], T[0],
+              Tlo[1], Thi[1], Tlo[0], Thi[0], ddeg, ndc, sel, len, span, span, amb);
     for (int pass = 0; pass < kFitPasses; ++pass) {
         const int a = pass & 1, b = a ^ 1;
         const bool last = pass + 1 == kFitPasses;
-        AD_LAUNCH(k_count_cand, cblocks, 256, 0, g->stream, info, pass == 0 ? nullptr : lists[a], L0,
-                  pass == 0 ? nullptr : len + a, goff, P, T[a], ndc, kFitCand, hist[a], cstar);
-        AD_LAUNCH(k_fit_advance, ablocks, 256, 0, g->stream, P, 0, last ? 1 : 0, st[a], st[b], hist[a], hist[b], T[a],
-                  T[b], Tlo[a], Thi[a], Tlo[b], Thi[b], ddeg, ndc, len + b, amb);
+        const FitSpan *sp = span + (size_t)pass * P;
+        AD_LAUNCH(k_fit_count, cblocks, 256, 0, g->stream, info, lists[0], lists[1], sel, len, goff, P, T[a], ndc, st[a],
+                  sp, pass, hist[a], cstar);
+        AD_LAUNCH(k_fit_advance, ablocks, 256, 0, g->stream, P, pass, last ? 1 : 0, st[a], st[b], hist[a], hist[b], T[a],
+                  T[b], Tlo[a], Thi[a], Tlo[b], Thi[b], ddeg, ndc, sel, len, sp, span + (size_t)(pass + 1) * P, amb);
         if (!last)
-            AD_LAUNCH(k_fit_compact, cblocks, 256, 0, g->stream, pass == 0 ? nullptr : lists[a], L0,
-                      pass == 0 ? nullptr : len + a, cstar, goff, P, st[b], lists[b], len + b);
+            AD_LAUNCH(k_fit_compact, cblocks, 256, 0, g->stream, lists[0], lists[1], sel, len, cstar, goff, P, st[a], sp,
+                      st[b], pass);
     }
     AD_TRY(copy_out(g, sh.data(), st[kFitPasses & 1], sizeof(FitState) * P));
     int amb_h = 0;
