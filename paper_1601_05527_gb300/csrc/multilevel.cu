@@ -540,21 +540,68 @@ static ad_status count_kept(ad_graph_t g, const uint8_t *keep, int64_t m, int64_
     return AD_OK;
 }
 
+// Finest edges behind every edge of a coarse level: mult of level l + 1 from mult
+// of level l (NULL at level 0: one each).
+__global__ void k_mult_up(const int64_t *f2c, const uint32_t *mult_f, int64_t m, uint32_t *mult_c) {
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < m && f2c[e] >= 0) atomicAdd(mult_c + f2c[e], mult_f ? mult_f[e] : 1u);
+}
+
+// sums over a level's edges: all of mult, and mult of the kept ones
+__global__ void k_mult_sums(const uint32_t *mult, const uint8_t *keep, int64_t m, unsigned long long *sums) {
+    unsigned long long a = 0, k = 0;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t x = mult ? mult[e] : 1u;
+        a += x;
+        k += keep[e] ? x : 0u;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        k += __shfl_xor_sync(0xffffffffu, k, o);
+    }
+    if ((threadIdx.x & 31) == 0 && a) {
+        atomicAdd(sums, a);
+        atomicAdd(sums + 1, k);
+    }
+}
+
+// mult of level `level` (device array owned by that level's graph; NULL for level 0)
+static ad_status level_multiplicity(ad_ml_t ml, int level, uint32_t **out) {
+    uint32_t *mult = nullptr;
+    for (int l = 0; l < level; ++l) {
+        ad_graph_t g = ml->lv[l].g, gc = ml->lv[l + 1].g;
+        uint32_t *next = nullptr;
+        AD_TRY(dalloc_t(gc, gc->m + 1, &next));
+        AD_CUDA_TRY(cudaMemsetAsync(next, 0, (gc->m + 1) * sizeof(uint32_t), g->stream));
+        if (g->m > 0) AD_LAUNCH(k_mult_up, nblk(g->m), 256, 0, g->stream, ml->lv[l].f2c, mult, g->m, next);
+        if (mult) dfree(g, mult);
+        mult = next;
+    }
+    *out = mult;
+    return AD_OK;
+}
+
 // Upward half of Alg. 6 with per-level keep fractions (index = level, 0 finest;
-// < 0 = level not sparsified).  keep0: device array [m_0].
-static ad_status ml_upward(ad_ml_t ml, const std::vector<double> &r, uint8_t *keep0, int64_t *kept) {
+// < 0 = level not sparsified).  keep0: device array [m_0].  With keep0 NULL only
+// the number of kept edges is wanted: the levels finer than `stop`, the finest
+// sparsified one, remove exactly the edges behind the removed edges of `stop`,
+// so the count follows from its mult and nothing finer is visited.
+static ad_status ml_upward(ad_ml_t ml, const std::vector<double> &r, uint8_t *keep0, int64_t *kept, int stop = 0,
+                           const uint32_t *mult = nullptr) {
     const int L = (int)ml->lv.size();
+    const bool count_only = keep0 == nullptr, trace = ml->trace && !count_only;
     uint8_t *keep_c = nullptr;
     ad_graph_t owner_c = nullptr;
-    for (int l = L - 1; l >= 0; --l) {
+    for (int l = L - 1; l >= stop; --l) {
         ad_graph_t g = ml->lv[l].g;
         ad_ml_s::Level &tv = ml->lv[l];
         uint8_t *keep = l == 0 ? keep0 : nullptr;
         if (!keep) AD_TRY(dalloc_t(g, g->m + 1, &keep));
-        if (ml->trace) AD_TRY(trace_buffers(tv));
+        if (trace) AD_TRY(trace_buffers(tv));
         if (l == L - 1) {
             AD_CUDA_TRY(cudaMemsetAsync(keep, 1, g->m > 0 ? g->m : 1, g->stream));
-            if (ml->trace && g->m > 0)
+            if (trace && g->m > 0)
                 AD_CUDA_TRY(cudaMemcpyAsync(tv.t_inh, keep, g->m, cudaMemcpyDeviceToDevice, g->stream));
             if (r[l] >= 0.0 && g->m > 0) {
                 int64_t k = 0;
@@ -563,7 +610,7 @@ static ad_status ml_upward(ad_ml_t ml, const std::vector<double> &r, uint8_t *ke
             }
         } else {
             if (g->m > 0) AD_LAUNCH(k_uncoarsen, nblk(g->m), 256, 0, g->stream, ml->lv[l].f2c, keep_c, g->m, keep);
-            if (ml->trace && g->m > 0)
+            if (trace && g->m > 0)
                 AD_CUDA_TRY(cudaMemcpyAsync(tv.t_inh, keep, g->m, cudaMemcpyDeviceToDevice, g->stream));
             if (r[l] >= 0.0 && g->m > 0) {
                 // ComputeAlgDist(G_f^s), then Sparsify(G_f^s)
@@ -585,7 +632,7 @@ static ad_status ml_upward(ad_ml_t ml, const std::vector<double> &r, uint8_t *ke
                         AD_CUDA_TRY(cudaMemsetAsync(keep, 0, g->m, g->stream));
                         AD_CUDA_TRY(cudaStreamSynchronize(sub->stream));
                         AD_LAUNCH(k_scatter_keep, nblk(ms), 256, 0, g->stream, s2f, ks, ms, keep);
-                        if (ml->trace) AD_LAUNCH(k_scatter_f32, nblk(ms), 256, 0, g->stream, s2f, sub->rho, ms, tv.t_rho);
+                        if (trace) AD_LAUNCH(k_scatter_f32, nblk(ms), 256, 0, g->stream, s2f, sub->rho, ms, tv.t_rho);
                         AD_CUDA_TRY(cudaStreamSynchronize(g->stream));
                     }
                 }
@@ -594,11 +641,24 @@ static ad_status ml_upward(ad_ml_t ml, const std::vector<double> &r, uint8_t *ke
                 AD_TRY(st);
             }
         }
-        if (ml->trace && g->m > 0)
+        if (trace && g->m > 0)
             AD_CUDA_TRY(cudaMemcpyAsync(tv.t_keep, keep, g->m, cudaMemcpyDeviceToDevice, g->stream));
         if (keep_c) dfree(owner_c, keep_c);
-        keep_c = l == 0 ? nullptr : keep;
+        keep_c = l == 0 && !count_only ? nullptr : keep;
         owner_c = g;
+    }
+    if (count_only) {   // keep_c: the kept edges of level `stop`
+        unsigned long long *sums = nullptr, v[2] = {0, 0};
+        AD_TRY(dalloc_t(owner_c, 2, &sums));
+        AD_CUDA_TRY(cudaMemsetAsync(sums, 0, 2 * sizeof(unsigned long long), owner_c->stream));
+        if (owner_c->m > 0)
+            AD_LAUNCH(k_mult_sums, (int)std::min<int64_t>(nblk(owner_c->m), (int64_t)owner_c->num_sms * 8), 256, 0,
+                      owner_c->stream, mult, keep_c, owner_c->m, sums);
+        AD_TRY(copy_out(owner_c, v, sums, sizeof(v)));
+        dfree(owner_c, sums);
+        dfree(owner_c, keep_c);
+        *kept = ml->lv[0].g->m - (int64_t)v[0] + (int64_t)v[1];   // edges inside aggregates are always kept
+        return AD_OK;
     }
     ml->have_trace = ml->trace;
     return count_kept(ml->lv[0].g, keep0, ml->lv[0].g->m, kept);
@@ -751,13 +811,18 @@ extern "C" ad_status ad_ml_sparsify(ad_ml_t ml, const double *ratios, int32_t n_
     } else {
         const int64_t K = (int64_t)std::floor(target_fraction * (double)g0->m + 0.5);
         double lo = 0.0, hi = 1.0;
+        int stop = 0;                                   // the finest sparsified level
+        while (stop < L - 1 && !(ratios[L - 1 - stop] >= 0.0)) ++stop;
+        uint32_t *mult = nullptr;
+        st = level_multiplicity(ml, stop, &mult);
         for (int it = 0; it < 20 && st == AD_OK; ++it) {
             const double mid = 0.5 * (lo + hi);
             for (int l = 0; l < L; ++l) r[l] = ratios[L - 1 - l] >= 0.0 ? mid : -1.0;
             int64_t c = 0;
-            st = ml_upward(ml, r, kd, &c);
+            st = ml_upward(ml, r, nullptr, &c, stop, mult);
             if (c >= K) hi = mid; else lo = mid;
         }
+        if (mult) dfree(ml->lv[stop].g, mult);
         if (st == AD_OK) {
             for (int l = 0; l < L; ++l) r[l] = ratios[L - 1 - l] >= 0.0 ? hi : -1.0;
             st = ml_upward(ml, r, kd, &kept);
