@@ -236,11 +236,27 @@ __global__ void k_degrees(const int64_t *rp, const int32_t *col, const float *w,
 // lane.  exact_out[i] records which case row i is (the seed rule relies on it).
 __device__ __forceinline__ int fp32_biased_exponent(float v) { return (int)((__float_as_uint(v) >> 23) & 0xffu); }
 
-__global__ void k_wdegrees(const int64_t *rp, const float *w, int64_t n, double *D, float *Dinv, uint8_t *exact_out) {
+// Rows longer than kLongDegreeRow are only listed (long_rows[0 .. *n_long)): one
+// warp would hold the launch up on a hub for milliseconds (R-MAT 22: 4.9 ms, all of
+// it hubs); k_wdegrees_long gives each a block.
+constexpr int64_t kLongDegreeRow = 2048;
+__device__ __forceinline__ bool sum_is_exact(int64_t d, int emax, int emin) {
+    int lg = 0;
+    while (((int64_t)1 << lg) < d) ++lg;   // ceil(log2 d)
+    // bits spanned by every partial sum: (emax - 127 + 1 + lg) - (max(emin, 1) - 150)
+    return d == 0 || emax - max(emin, 1) + lg + 24 <= 53;
+}
+
+__global__ void k_wdegrees(const int64_t *rp, const float *w, int64_t n, double *D, float *Dinv, uint8_t *exact_out,
+                           int32_t *long_rows, unsigned int *n_long) {
     const int lane = threadIdx.x & 31;
     const int64_t W = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += W) {
         const int64_t b = rp[i], e = rp[i + 1];
+        if (e - b > kLongDegreeRow) {
+            if (lane == 0) long_rows[atomicAdd(n_long, 1u)] = (int32_t)i;
+            continue;
+        }
         double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;   // four independent loads in flight per lane
         int emax = 0, emin = 255;
         int64_t p = b + lane;
@@ -268,10 +284,7 @@ __global__ void k_wdegrees(const int64_t *rp, const float *w, int64_t n, double 
             emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
             emin = min(emin, __shfl_xor_sync(0xffffffffu, emin, o));
         }
-        int lg = 0;
-        while (((int64_t)1 << lg) < e - b) ++lg;   // ceil(log2 d)
-        // bits spanned by every partial sum: (emax - 127 + 1 + lg) - (max(emin, 1) - 150)
-        const bool exact = e == b || emax - max(emin, 1) + lg + 24 <= 53;
+        const bool exact = sum_is_exact(e - b, emax, emin);
         if (lane == 0) {
             if (!exact) {   // the plain definition's order, one entry after the other
                 s = 0.0;
@@ -281,6 +294,85 @@ __global__ void k_wdegrees(const int64_t *rp, const float *w, int64_t n, double 
             Dinv[i] = s > 0.0 ? (float)(1.0 / s) : 0.f;
             exact_out[i] = exact ? 1 : 0;
         }
+    }
+}
+
+// The listed long rows, a block each: the same sum where it is exact, otherwise
+// one after the other in CSR order by one thread, from shared memory.
+constexpr int kLongDegreeThreads = 512;
+__global__ void __launch_bounds__(kLongDegreeThreads) k_wdegrees_long(const int64_t *rp, const float *w,
+                                                                      const int32_t *rows, const unsigned int *n_rows,
+                                                                      double *D, float *Dinv, uint8_t *exact_out) {
+    constexpr int T = kLongDegreeThreads, NW = T / 32, kTile = 4 * T;
+    __shared__ double ssum[NW];
+    __shared__ int smax[NW], smin[NW];
+    __shared__ float tile[kTile];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned int count = *n_rows;
+    for (unsigned int t = blockIdx.x; t < count; t += gridDim.x) {
+        const int64_t i = rows[t], b = rp[i], e = rp[i + 1];
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+        int emax = 0, emin = 255;
+        auto take = [&](float v, double &s) {
+            s += (double)v;
+            emax = max(emax, fp32_biased_exponent(v));
+            emin = min(emin, fp32_biased_exponent(v));
+        };
+        int64_t p = b + threadIdx.x;
+        for (; p + 3 * T < e; p += 4 * T) {
+            const float w0 = w[p], w1 = w[p + T], w2 = w[p + 2 * T], w3 = w[p + 3 * T];
+            take(w0, s0);
+            take(w1, s1);
+            take(w2, s2);
+            take(w3, s3);
+        }
+        for (; p < e; p += T) take(w[p], s0);
+        double s = (s0 + s1) + (s2 + s3);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+            emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+            emin = min(emin, __shfl_xor_sync(0xffffffffu, emin, o));
+        }
+        if (lane == 0) {
+            ssum[warp] = s;
+            smax[warp] = emax;
+            smin[warp] = emin;
+        }
+        __syncthreads();
+        s = 0.0;
+        for (int k = 0; k < NW; ++k) {
+            s += ssum[k];
+            emax = max(emax, smax[k]);
+            emin = min(emin, smin[k]);
+        }
+        const bool exact = sum_is_exact(e - b, emax, emin);
+        if (!exact) {   // the plain definition's order
+            s = 0.0;
+            for (int64_t q0 = b; q0 < e; q0 += kTile) {
+                __syncthreads();
+                for (int k = threadIdx.x; k < kTile && q0 + k < e; k += T) tile[k] = w[q0 + k];
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    const int cnt = (int)min((int64_t)kTile, e - q0);
+                    int k = 0;
+                    for (; k + 8 <= cnt; k += 8) {
+                        float v[8];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) v[u] = tile[k + u];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) s += (double)v[u];
+                    }
+                    for (; k < cnt; ++k) s += (double)tile[k];
+                }
+            }
+        }
+        if (threadIdx.x == 0) {
+            D[i] = s;
+            Dinv[i] = s > 0.0 ? (float)(1.0 / s) : 0.f;
+            exact_out[i] = exact ? 1 : 0;
+        }
+        __syncthreads();
     }
 }
 
@@ -381,10 +473,18 @@ ad_status recompute_degrees(ad_graph_t g) {
     const int64_t tblocks = std::min<int64_t>((g->n + 255) / 256 + 1, (int64_t)g->num_sms * 16);
     AD_LAUNCH(k_degrees, (int)tblocks, 256, 0, g->stream, g->rp, g->col, g->w, g->n, g->D, g->Dinv, g->upos,
               ucount);
+    int32_t *lrows = nullptr;
     if (g->w) {
         const int64_t wblocks = std::min<int64_t>((g->n + 7) / 8 + 1, (int64_t)g->num_sms * 64);
         if (!g->dexact) AD_TRY(dalloc_t(g, g->n + 1, &g->dexact));
-        AD_LAUNCH(k_wdegrees, (int)wblocks, 256, 0, g->stream, g->rp, g->w, g->n, g->D, g->Dinv, g->dexact);
+        const int64_t cap = g->nnz / kLongDegreeRow + 1;   // more rows cannot be that long
+        AD_TRY(dalloc_t(g, cap + 1, &lrows));
+        unsigned int *n_long = reinterpret_cast<unsigned int *>(lrows + cap);
+        AD_CUDA_TRY(cudaMemsetAsync(n_long, 0, sizeof(unsigned int), g->stream));
+        AD_LAUNCH(k_wdegrees, (int)wblocks, 256, 0, g->stream, g->rp, g->w, g->n, g->D, g->Dinv, g->dexact, lrows, n_long);
+        if (cap > 1)
+            AD_LAUNCH(k_wdegrees_long, (int)std::min<int64_t>(cap, (int64_t)g->num_sms * 4), kLongDegreeThreads, 0,
+                      g->stream, g->rp, g->w, lrows, n_long, g->D, g->Dinv, g->dexact);
     }
     int64_t m = 0;
     ad_status st = exclusive_scan_i64(g, ucount, g->eoff, g->n, &m);
@@ -392,6 +492,7 @@ ad_status recompute_degrees(ad_graph_t g) {
     AD_TRY(st);
     AD_CUDA_TRY(cudaMemcpyAsync(g->eoff + g->n, &m, sizeof(int64_t), cudaMemcpyHostToDevice, g->stream));
     AD_CUDA_TRY(cudaStreamSynchronize(g->stream));
+    if (lrows) dfree(g, lrows);
     g->m = m;
     return compute_anchors(g);
 }
