@@ -79,14 +79,47 @@ static ad_status make_tiles(ad_graph_t g, Tiles &t) {
     return AD_OK;
 }
 
+// f(score[e]) for every e of a tile [s, e1) by the block, in no particular order:
+// 16-byte loads, four in flight per thread, where the tile starts on a 16-byte
+// boundary (a caller's scores and the graphs of a batch need not), 4-byte ones
+// otherwise.  The passes of the radix select are reads of 4 bytes per edge.
+template <typename F>
+__device__ __forceinline__ void for_tile(const float *score, int64_t s, int64_t e1, F f) {
+    if ((reinterpret_cast<uintptr_t>(score + s) & 15) == 0 && e1 - s == kTile) {
+        const float4 *v = reinterpret_cast<const float4 *>(score + s);
+        constexpr int N = kTileItems / 4;
+        float4 x[N];
+#pragma unroll
+        for (int u = 0; u < N; ++u) x[u] = __ldg(v + u * kTileThreads + threadIdx.x);
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            f(x[u].x);
+            f(x[u].y);
+            f(x[u].z);
+            f(x[u].w);
+        }
+    } else {
+        for (int64_t e = s + threadIdx.x; e < e1; e += kTileThreads) f(score[e]);
+    }
+}
+
 // ----------------------------------------------------------------------------
 // Score validation: every score finite and >= 0.
 // ----------------------------------------------------------------------------
 __global__ void k_check_scores(const float *s, int64_t m, unsigned long long *bad) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        const float x = s[e];
+    auto check = [&](float x, int64_t e) {
         if (!(x >= 0.f) || !isfinite(x)) atomicMin(bad, (unsigned long long)e);
+    };
+    const int64_t step = (int64_t)gridDim.x * blockDim.x, t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t quads = (reinterpret_cast<uintptr_t>(s) & 15) == 0 ? m / 4 : 0;
+    for (int64_t q = t; q < quads; q += step) {
+        const float4 x = __ldg(reinterpret_cast<const float4 *>(s) + q);
+        check(x.x, 4 * q);
+        check(x.y, 4 * q + 1);
+        check(x.z, 4 * q + 2);
+        check(x.w, 4 * q + 3);
     }
+    for (int64_t e = 4 * quads + t; e < m; e += step) check(s[e], e);
 }
 
 // ----------------------------------------------------------------------------
@@ -101,10 +134,10 @@ __global__ void k_sel_hist(const float *score, int desc, const int32_t *tg, cons
     const SelState s = st[gph];
     if (s.k_rem > 0) {
         const uint32_t dmask = (1u << bits) - 1u;
-        for (int64_t e = ts[blockIdx.x] + threadIdx.x; e < te[blockIdx.x]; e += blockDim.x) {
-            const uint32_t k = score_key(score[e], desc);
+        for_tile(score, ts[blockIdx.x], te[blockIdx.x], [&](float x) {
+            const uint32_t k = score_key(x, desc);
             if ((k & hi_mask) == s.prefix) atomicAdd(&h[(k >> shift) & dmask], 1u);
-        }
+        });
     }
     __syncthreads();
     for (int b = threadIdx.x; b < (1 << bits); b += blockDim.x)
@@ -165,8 +198,8 @@ __global__ void k_sel_ties(const float *score, int desc, const int32_t *tg, cons
     const SelState s = st[gph];
     int64_t c = 0;
     if (s.k_rem > 0)
-        for (int64_t e = ts[blockIdx.x] + threadIdx.x; e < te[blockIdx.x]; e += blockDim.x)
-            c += (score_key(score[e], desc) == s.prefix) ? 1 : 0;
+        for_tile(score, ts[blockIdx.x], te[blockIdx.x],
+                 [&](float x) { c += (score_key(x, desc) == s.prefix) ? 1 : 0; });
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = c;
     __syncthreads();
@@ -186,9 +219,23 @@ __global__ void k_sel_write(const float *score, int desc, const int32_t *tg, con
     const int64_t e0 = ts[blockIdx.x] + (int64_t)threadIdx.x * kTileItems, e1 = te[blockIdx.x];
     uint32_t k[kTileItems];
     int64_t my = 0;
+    // a thread's 16 edges by 16-byte loads and one 16-byte store, where they are whole and aligned
+    const bool whole = e0 + kTileItems <= e1;
+    if (whole && (reinterpret_cast<uintptr_t>(score + e0) & 15) == 0) {
+#pragma unroll
+        for (int u = 0; u < kTileItems / 4; ++u) {
+            const float4 x = __ldg(reinterpret_cast<const float4 *>(score + e0) + u);
+            k[4 * u] = score_key(x.x, desc);
+            k[4 * u + 1] = score_key(x.y, desc);
+            k[4 * u + 2] = score_key(x.z, desc);
+            k[4 * u + 3] = score_key(x.w, desc);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < kTileItems; ++i) k[i] = (e0 + i < e1) ? score_key(score[e0 + i], desc) : 0xffffffffu;
+    }
 #pragma unroll
     for (int i = 0; i < kTileItems; ++i) {
-        k[i] = (e0 + i < e1) ? score_key(score[e0 + i], desc) : 0xffffffffu;
         my += (e0 + i < e1 && s.k_rem > 0 && k[i] == s.prefix) ? 1 : 0;
     }
     // block exclusive scan of tie counts (threads own consecutive edges)
@@ -210,25 +257,41 @@ __global__ void k_sel_write(const float *score, int desc, const int32_t *tg, con
     }
     __syncthreads();
     int64_t rank = tie_off[blockIdx.x] - tie_off[first_tile[gph]] + (warp > 0 ? sh[warp - 1] : 0) + x - my;
+    uint32_t word[kTileItems / 4] = {};
 #pragma unroll
     for (int i = 0; i < kTileItems; ++i) {
         if (e0 + i >= e1) break;
-        uint8_t kp = 0;
+        uint32_t kp = 0;
         if (s.K >= s.m) kp = 1;
         else if (s.K > 0) {
             if (k[i] < s.prefix) kp = 1;
             else if (k[i] == s.prefix) { kp = rank < s.k_rem ? 1 : 0; ++rank; }
         }
-        keep[e0 + i] = kp;
+        word[i / 4] |= kp << (8 * (i % 4));
+    }
+    if (whole && (reinterpret_cast<uintptr_t>(keep + e0) & 15) == 0) {
+        *reinterpret_cast<uint4 *>(keep + e0) = make_uint4(word[0], word[1], word[2], word[3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < kTileItems; ++i)
+            if (e0 + i < e1) keep[e0 + i] = (uint8_t)(word[i / 4] >> (8 * (i % 4)));
     }
 }
+static_assert(kTileItems == 16, "k_sel_write packs a thread's 16 flags");
 
 // ----------------------------------------------------------------------------
 // Per-node ranks
 // ----------------------------------------------------------------------------
-// The ranking key of a CSR entry: the caller's array, or the score of its edge
-// (read where the entry is ranked: a pass that wrote the keys first cost a read
-// and a write of 4 bytes per entry and a launch).
+__global__ void k_entry_keys(const int64_t *eid, int64_t nnz, const float *score, uint32_t *ekey) {
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x)
+        ekey[p] = score_key(score[eid[p]], 0);
+}
+
+// The ranking key of a CSR entry: an array, or the score of its edge, read where
+// the entry is ranked.  The counting kernels of short rows take the latter in
+// their stride (128 Watts-Strogatz graphs: ranks 1.41 -> 1.61 ms, the pass that wrote
+// the keys, 0.41 ms, gone); the sorts of longer rows wait on the two dependent loads
+// (R-MAT 20: 0.17 ms more in the sorts against a pass of 0.12 ms).
 struct KeySrc {
     const uint32_t *ekey;    // [nnz], or
     const int64_t *eid;      // edge of every entry and
@@ -773,7 +836,7 @@ __device__ __forceinline__ bool fit_all_known(const FitState *st, const FitSpan 
 // State, tables, ends and histograms are double-buffered by pass parity.
 // pass: the one just counted (-1: none, the state is the initial one); list
 // selectors and lengths are kept per pass: sel 0: all edges, 1 and 2: the lists.
-__global__ void __launch_bounds__(256) k_fit_advance(int P, int pass, int last, const FitState *st_old, FitState *st_new,
+__global__ void __launch_bounds__(64) k_fit_advance(int P, int pass, int last, const FitState *st_old, FitState *st_new,
                               const unsigned long long *hist, unsigned long long *hist_next, const int32_t *T_cur,
                               int32_t *T_next, const int32_t *Tlo_old, const int32_t *Thi_old, int32_t *Tlo_new,
                               int32_t *Thi_new, const int64_t *ddeg, int32_t ndc, int32_t *sel, int64_t *len,
@@ -1225,7 +1288,19 @@ static ad_status per_node_info(ad_graph_t g, const float *score, ad_mode mode, i
     RankOut out;
     out.asc = asc ? ranks : nullptr;
     out.desc = desc ? ranks + (nnz + 1) : nullptr;
-    AD_TRY(entry_ranks(g, c, KeySrc{nullptr, g->eid, score}, out));
+    // a pass that writes the keys where rows of more than 32 entries, which are sorted,
+    // hold a quarter of the entries or more (counted from below: class size x smallest row)
+    static const int64_t kSmallest[10] = {0, 0, 0, 33, 65, 129, 257, 513, kSortCap + 1, kSortCapLarge + 1};
+    int64_t sorted_entries = 0;
+    for (int k = 3; k < 10; ++k) sorted_entries += c->nrows[k] * kSmallest[k];
+    KeySrc keys{nullptr, g->eid, score};
+    if (4 * sorted_entries >= nnz && nnz > 0) {
+        AD_TRY(ensure(g, c->ekey, sizeof(uint32_t) * (nnz + 1)));
+        uint32_t *ekey = static_cast<uint32_t *>(c->ekey.ptr);
+        AD_LAUNCH(k_entry_keys, g->num_sms * 16, 256, 0, g->stream, g->eid, nnz, score, ekey);
+        keys.ekey = ekey;
+    }
+    AD_TRY(entry_ranks(g, c, keys, out));
     if (g->m > 0)
         AD_LAUNCH(k_info, g->num_sms * 16, 256, 0, g->stream, c->epos, g->mirror, g->erow, g->col, g->deg_class, g->m,
                   out.asc, out.desc, info_asc, info_desc);
@@ -1510,10 +1585,12 @@ static ad_status fit_multi(ad_graph_t g, const int4 *info, int nsets, double fra
                                 g->stream));
     AD_TRY(copy_in(g, len, &L0, sizeof(int64_t)));
     const int big = g->num_sms * 16;
-    const int ablocks = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)tsz + 255) / 256, big));
+    // blocks of 64: a table entry is an FP64 pow on this part's narrow FP64 pipe, so small
+    // tables are spread over more SMs (the 462 launches of a multilevel call: 5.4 -> 4.9 ms)
+    const int ablocks = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)tsz + 63) / 64, 4 * big));
     const int cblocks = (int)std::max<int64_t>(1, std::min<int64_t>((L0 + 255) / 256, big));
     // initial state, ends and the tables of pass 0
-    AD_LAUNCH(k_fit_advance, ablocks, 256, 0, g->stream, P, -1, 0, stb + 2 * P, st[0], hist[1], hist[0], T[1], T[0],
+    AD_LAUNCH(k_fit_advance, ablocks, 64, 0, g->stream, P, -1, 0, stb + 2 * P, st[0], hist[1], hist[0], T[1], T[0],
               Tlo[1], Thi[1], Tlo[0], Thi[0], ddeg, ndc, sel, len, span, span, amb);
     for (int pass = 0; pass < kFitPasses; ++pass) {
         const int a = pass & 1, b = a ^ 1;
@@ -1521,7 +1598,7 @@ static ad_status fit_multi(ad_graph_t g, const int4 *info, int nsets, double fra
         const FitSpan *sp = span + (size_t)pass * P;
         AD_LAUNCH(k_fit_count, cblocks, 256, 0, g->stream, info, lists[0], lists[1], sel, len, goff, P, T[a], ndc, st[a],
                   sp, pass, hist[a], cstar);
-        AD_LAUNCH(k_fit_advance, ablocks, 256, 0, g->stream, P, pass, last ? 1 : 0, st[a], st[b], hist[a], hist[b], T[a],
+        AD_LAUNCH(k_fit_advance, ablocks, 64, 0, g->stream, P, pass, last ? 1 : 0, st[a], st[b], hist[a], hist[b], T[a],
                   T[b], Tlo[a], Thi[a], Tlo[b], Thi[b], ddeg, ndc, sel, len, sp, span + (size_t)(pass + 1) * P, amb);
         if (!last)
             AD_LAUNCH(k_fit_compact, cblocks, 256, 0, g->stream, lists[0], lists[1], sel, len, cstar, goff, P, st[a], sp,
