@@ -189,20 +189,21 @@ __global__ void k_aggregate(const int64_t *rp, const int32_t *col, const int64_t
 // ----------------------------------------------------------------------------
 // Galerkin coarse graph
 // ----------------------------------------------------------------------------
-__global__ void k_coarse_pairs(const int64_t *rp, const int32_t *col, const float *w, const int64_t *upos,
-                               const int64_t *eoff, const int32_t *agg, int64_t n, uint8_t *inter, uint64_t *key,
+// a thread per CSR entry (most rows have a handful of upper entries, which a warp
+// per row left nearly empty); the upper ones write
+__global__ void k_coarse_pairs(const int32_t *erow, const int32_t *col, const float *w, const int64_t *upos,
+                               const int64_t *eoff, const int32_t *agg, int64_t nnz, uint8_t *inter, uint64_t *key,
                                double *we) {
-    const int lane = threadIdx.x & 31;
-    const int64_t W = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += W)
-        for (int64_t p = upos[i] + lane; p < rp[i + 1]; p += 32) {
-            const int64_t e = eoff[i] + (p - upos[i]);
-            const int32_t I = agg[i], J = agg[col[p]];
-            inter[e] = (I != J && I >= 0 && J >= 0) ? 1 : 0;
-            const uint64_t a = (uint64_t)min(I, J), b = (uint64_t)max(I, J);
-            key[e] = (a << 32) | b;
-            we[e] = w ? (double)w[p] : 1.0;
-        }
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t i = erow[p], j = col[p];
+        if (j <= i) continue;
+        const int64_t e = eoff[i] + (p - upos[i]);
+        const int32_t I = agg[i], J = agg[j];
+        inter[e] = (I != J && I >= 0 && J >= 0) ? 1 : 0;
+        const uint64_t a = (uint64_t)min(I, J), b = (uint64_t)max(I, J);
+        key[e] = (a << 32) | b;
+        we[e] = w ? (double)w[p] : 1.0;
+    }
 }
 
 __global__ void k_gather_keys(const uint64_t *key, const int64_t *idx, int64_t n, uint64_t *out) {
@@ -346,8 +347,8 @@ static ad_status coarsen_level(ad_graph_t g, const float *score, double Q, int32
     AD_TRY(dalloc_t(g, m + 1, &key));
     AD_TRY(dalloc_t(g, m + 1, &we));
     if (m > 0)
-        AD_LAUNCH(k_coarse_pairs, (int)wblocks, 256, 0, g->stream, g->rp, g->col, g->w, g->upos, g->eoff, agg, n, inter,
-                  key, we);
+        AD_LAUNCH(k_coarse_pairs, g->num_sms * 16, 256, 0, g->stream, g->erow, g->col, g->w, g->upos, g->eoff, agg, g->nnz,
+                  inter, key, we);
     int64_t *fine = nullptr;
     int64_t mi = 0;
     AD_TRY(compact_flags(g, inter, m, &fine, &mi));
@@ -436,8 +437,11 @@ __global__ void k_sub_count(const int64_t *rp, const int64_t *eid, const uint8_t
     const int64_t W = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += W) {
         int64_t c = 0;
-        for (int64_t p = rp[i] + lane; p < rp[i + 1]; p += 32)
-            c += keep[eid[p]] ? 1 : 0;
+        const int64_t end = rp[i + 1];
+        for (int64_t p0 = rp[i] + lane; p0 < end; p0 += 128) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) c += p0 + 32 * u < end && keep[eid[p0 + 32 * u]] ? 1 : 0;
+        }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
         if (lane == 0) cnt[i] = c;
@@ -450,17 +454,25 @@ __global__ void k_sub_fill(const int64_t *rp, const int32_t *col, const float *w
     const int64_t W = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += W) {
         int64_t out = rps[i];
-        for (int64_t base = rp[i]; base < rp[i + 1]; base += 32) {
-            const int64_t p = base + lane;
-            bool k = false;
-            if (p < rp[i + 1]) k = keep[eid[p]] != 0;
-            const unsigned b = __ballot_sync(0xffffffffu, k);
-            if (k) {
-                const int64_t q = out + __popc(b & ((1u << lane) - 1u));
-                cols[q] = col[p];
-                if (ws) ws[q] = w[p];
+        const int64_t end = rp[i + 1];
+        for (int64_t base = rp[i]; base < end; base += 128) {   // four chunks' flags in flight
+            bool k[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t p = base + 32 * u + lane;
+                k[u] = p < end && keep[eid[p]] != 0;
             }
-            out += __popc(b);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t p = base + 32 * u + lane;
+                const unsigned b = __ballot_sync(0xffffffffu, k[u]);
+                if (k[u]) {
+                    const int64_t q = out + __popc(b & ((1u << lane) - 1u));
+                    cols[q] = col[p];
+                    if (ws) ws[q] = w[p];
+                }
+                out += __popc(b);
+            }
         }
     }
 }
