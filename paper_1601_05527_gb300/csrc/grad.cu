@@ -14,14 +14,11 @@
 //     xbar_{t-1} = (1-omega) ybar_t + omega W (D^-1 ybar_t)        (W symmetric)
 //     dL/dw_ij  += omega ybar_t,i . (x_{t-1,j} - avg_i) / D_i,   avg_i = D_i^-1 sum_l w_il x_{t-1,l}
 // and in the stored frame x_{t-1,j} - avg_i = a_{t-1} (s_{t-1,j} - sigma_i) with
-// sigma_i = D_i^-1 sum_l w_il s_{t-1,l}.  With U = D^-1 ybar_t the kernels keep,
-// for the two entries p = (i, j), q = (j, i) of every edge,
-//     G_p = sum_t (a_{t-1} U_i) . s_{t-1,j},   G_q = sum_t (a_{t-1} s_{t-1,i}) . U_j;
-// both come from one visit of the edge's upper entry, which has row i in
-// registers and fetches [U_j | s_j].  The sigma term needs no gather of its own:
-// sum_t a_{t-1} U_i . sigma_i = C_i = D_i^-1 sum_l w_il G_il, taken once at the end, and
-// dL/dw_e = omega (G_p - C_i + G_q - C_j).  All sums are in a fixed order (no
-// floating-point atomics), G and C in FP64.
+// sigma_i = D_i^-1 sum_l w_il s_{t-1,l}.  Per CSR entry p = (i, j) the kernels
+// accumulate G_p = sum_t v_i . s_{t-1,j} and per row C_i = sum_t v_i . sigma_i with
+// v_i = ybar_t,i * a_{t-1}; then dL/dw_e = omega (G_p - C_i) / D_i + omega (G_q - C_j) / D_j
+// for the two entries p = (i, j), q = (j, i) of edge e.  All sums are in a fixed
+// order (no floating-point atomics), G and C in FP64.
 //
 // Memory: the stored vectors after sweeps 0, c, 2c, ... (c = ceil(sqrt k)) are
 // kept by the forward; each segment of c sweeps is recomputed from its
@@ -115,18 +112,21 @@ struct BwArgs {
     const float *rho, *rhobar;
     const float *a_k;            // [stride] per-vector scale of the last iterate (device)
     // sweep backward
-    const float *Z;              // rows [U_i | s_{t-1,i}], 2 * stride floats each
+    const float *U;              // D^-1 ybar_t
+    const float *Sprev;          // stored s_{t-1}
+    int32_t gpitch;              // row pitch (floats) of U and Sprev in the adjoint gather
     const float *Ybar;           // ybar_t
     const float *a_prev;         // [stride] a_{t-1} (device; nullptr: 1, for t = 1)
     const float *Sk;             // stored s_k (distance backward input)
-    const int64_t *upos, *eoff;
     float *xbar_out;
-    double *G;                   // [m][2]: G_p and G_q of every edge
+    double *G;                   // [nnz]
+    double *C;                   // [n]
     float *part;                 // [n_big][2][stride]
     // plan
     const int32_t *big_row, *big_chunk, *medium_row, *small_row;
     uint32_t *big_counter;
-    int64_t n_big, n_medium, n_small_rows, n_tasks, n_wide;
+    int64_t n_big, n_medium, n_small_rows, n_tasks;
+    int mode;                    // 0: distance backward, 1: sweep backward
 };
 
 template <int CPL>
@@ -135,13 +135,23 @@ __device__ __forceinline__ void ld4(const float *base, int64_t row, int stride, 
     out[0] = f.x; out[1] = f.y; out[2] = f.z; out[3] = f.w;
 }
 
-// ---- distance backward: xbar_k from rhobar ----------------------------------
-// One row (or chunk of a row) p in [p0, p1) processed by the warp (G groups
-// over neighbours) or by one group (G = 1 group, gstride = 1):
-// acc_a = sum c_p s_j, acc_b = sum c_p (scalar in slot 0)
 template <int LPR, int CPL>
-__device__ __forceinline__ void bw_gather(const BwArgs &a, int64_t p0, int64_t p1, int first, int gstride, int gl,
-                                          float (&acc_a)[CPL * 4], float (&acc_b)[CPL * 4]) {
+__device__ __forceinline__ void bw_gather_adjoint(const BwArgs &a, int64_t p0, int64_t p1, int first, int gstride,
+                                                  int gl, unsigned gmask, const float (&v)[CPL * 4],
+                                                  float (&acc_a)[CPL * 4], float (&acc_b)[CPL * 4]);
+
+// One row (or chunk of a row) p in [p0, p1) processed by the warp (G groups
+// over neighbours) or by one group (G = 1 group, gstride = 1).
+//   mode 0: acc_a = sum c_p s_j, acc_b = sum c_p (scalar in slot 0)
+//   mode 1: acc_a = sum w U_j, acc_b = sum w s_j, G_p += v_i . s_j (bw_gather_adjoint)
+template <int LPR, int CPL>
+__device__ __forceinline__ void bw_gather(const BwArgs &a, int64_t row, int64_t p0, int64_t p1, int first, int gstride,
+                                          int gl, unsigned gmask, const float (&v)[CPL * 4], float (&acc_a)[CPL * 4],
+                                          float (&acc_b)[CPL * 4]) {
+    if (a.mode == 1) {
+        bw_gather_adjoint<LPR, CPL>(a, p0, p1, first, gstride, gl, gmask, v, acc_a, acc_b);
+        return;
+    }
     for (int64_t p = p0 + first; p < p1; p += gstride) {
         const int32_t j = __ldg(a.col + p);
         {
@@ -163,12 +173,118 @@ __device__ __forceinline__ void bw_gather(const BwArgs &a, int64_t p0, int64_t p
     }
 }
 
-// xbar_k,i = a_k (sum_j c_ij s_i - sum_j c_ij s_j)
+// mode 1 in batches of kBwUB neighbours per group: all their loads are issued
+// before any is used, and the per-entry dots are summed over the group's lanes
+// together (group_sums)
+#ifndef AD_BW_UB
+#define AD_BW_UB 8            // neighbours in flight per group (measured at R-MAT 22: 8 with 3 CTAs per SM fastest)
+#endif
+#ifndef AD_BW_GPF
+#define AD_BW_GPF 1
+#endif
+
+constexpr int kBwUB = AD_BW_UB;
 template <int LPR, int CPL>
-__device__ __forceinline__ void bw_finish(const BwArgs &a, int64_t row, int gl, const float (&own)[CPL * 4],
+__device__ __forceinline__ void bw_gather_adjoint(const BwArgs &a, int64_t p0, int64_t p1, int first, int gstride,
+                                                  int gl, unsigned gmask, const float (&v)[CPL * 4],
+                                                  float (&acc_a)[CPL * 4], float (&acc_b)[CPL * 4]) {
+    constexpr int UB = kBwUB;
+    constexpr int NH = UB / LPR > 0 ? UB / LPR : 1;
+    constexpr int WS = LPR > UB ? LPR / UB : 1;   // lanes per entry that hold the same dot
+    const bool writer = gl % WS == 0;
+    // the entries whose dots this lane will hold after group_sums
+    int which = 0;
+#pragma unroll
+    for (int o = LPR / 2, c = UB; o >= 1; o >>= 1)
+        if (c > 1) {
+            if (gl & o) which += c / 2;
+            c >>= 1;
+        }
+    for (int64_t pb = p0 + first; pb < p1; pb += (int64_t)gstride * UB) {
+        int32_t jn[UB];
+        float wt[UB];
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+            const int64_t p = pb + (int64_t)u * gstride;
+            const bool ok = p < p1;
+            jn[u] = ok ? __ldg(a.col + p) : 0;
+            wt[u] = ok ? (a.w ? __ldg(a.w + p) : 1.f) : 0.f;
+        }
+#if AD_BW_GPF
+        // the accumulators of those entries, loaded with the rows so that their latency overlaps
+        double gold[NH];
+#pragma unroll
+        for (int i = 0; i < NH; ++i) {
+            const int64_t p = pb + (int64_t)(which + i) * gstride;
+            gold[i] = (writer && p < p1) ? __ldcg(a.G + p) : 0.0;
+        }
+#endif
+        float4 uu[UB][CPL], ss[UB][CPL];
+#pragma unroll
+        for (int u = 0; u < UB; ++u)
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) {
+                const int q = gl + c * LPR;
+                const bool ok = pb + (int64_t)u * gstride < p1 && q < a.nchunks;
+                uu[u][c] = ok ? __ldg(reinterpret_cast<const float4 *>(a.U + (int64_t)jn[u] * a.gpitch) + q)
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+                ss[u][c] = ok ? __ldg(reinterpret_cast<const float4 *>(a.Sprev + (int64_t)jn[u] * a.gpitch) + q)
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        float dot[UB];
+#pragma unroll
+        for (int u = 0; u < UB; ++u) {
+            dot[u] = 0.f;
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) {
+                const float uf[4] = {uu[u][c].x, uu[u][c].y, uu[u][c].z, uu[u][c].w};
+                const float sf[4] = {ss[u][c].x, ss[u][c].y, ss[u][c].z, ss[u][c].w};
+#pragma unroll
+                for (int e4 = 0; e4 < 4; ++e4) {
+                    acc_a[c * 4 + e4] = fmaf(wt[u], uf[e4], acc_a[c * 4 + e4]);
+                    acc_b[c * 4 + e4] = fmaf(wt[u], sf[e4], acc_b[c * 4 + e4]);
+                    dot[u] = fmaf(v[c * 4 + e4], sf[e4], dot[u]);
+                }
+            }
+        }
+        int w2 = 0;
+        group_sums<LPR, UB>(dot, gl, gmask, w2);
+#pragma unroll
+        for (int i = 0; i < NH; ++i) {
+            const int64_t p = pb + (int64_t)(which + i) * gstride;
+#if AD_BW_GPF
+            if (writer && p < p1) a.G[p] = gold[i] + (double)dot[i];
+#else
+            if (writer && p < p1) a.G[p] += (double)dot[i];
+#endif
+        }
+    }
+}
+
+template <int LPR, int CPL>
+__device__ __forceinline__ void bw_finish(const BwArgs &a, int64_t row, int gl, unsigned gmask,
+                                          const float (&v)[CPL * 4], const float (&own)[CPL * 4],
                                           const float (&acc_a)[CPL * 4], const float (&acc_b)[CPL * 4]) {
     float *xo = a.xbar_out + row * (int64_t)a.stride;
-    const float csum = acc_b[0];
+    if (a.mode == 0) {
+        // xbar_k,i = a_k (sum_j c_ij s_i - sum_j c_ij s_j)
+        const float csum = acc_b[0];
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) {
+            const int q = gl + c * LPR;
+            if (q < a.nchunks) {
+#pragma unroll
+                for (int e4 = 0; e4 < 4; ++e4) {
+                    const int r = q * 4 + e4;
+                    xo[r] = (r < a.R ? __ldg(a.a_k + r) : 0.f) * (csum * own[c * 4 + e4] - acc_a[c * 4 + e4]);
+                }
+            }
+        }
+        return;
+    }
+    const float dinv = __ldg(a.Dinv + row);
+    const float om = a.omega, om1 = 1.f - a.omega;
+    float cdot = 0.f;
 #pragma unroll
     for (int c = 0; c < CPL; ++c) {
         const int q = gl + c * LPR;
@@ -176,34 +292,46 @@ __device__ __forceinline__ void bw_finish(const BwArgs &a, int64_t row, int gl, 
 #pragma unroll
             for (int e4 = 0; e4 < 4; ++e4) {
                 const int r = q * 4 + e4;
-                xo[r] = (r < a.R ? __ldg(a.a_k + r) : 0.f) * (csum * own[c * 4 + e4] - acc_a[c * 4 + e4]);
+                xo[r] = fmaf(om1, own[c * 4 + e4], om * acc_a[c * 4 + e4]);
+                cdot = fmaf(v[c * 4 + e4], dinv * acc_b[c * 4 + e4], cdot);
             }
         }
     }
+#pragma unroll
+    for (int off = 1; off < LPR; off <<= 1) cdot += __shfl_xor_sync(gmask, cdot, off);
+    if (gl == 0) a.C[row] += (double)cdot;
 }
 
-// a row of floats (pitch floats apart), the lane's chunks
+// own values of row i: mode 0 -> s_k,i ; mode 1 -> ybar_t,i (v = ybar * a_{t-1})
 template <int LPR, int CPL>
-__device__ __forceinline__ void bw_row(const float *base, int64_t row, int pitch, int nchunks, int gl, float (&own)[CPL * 4]) {
+__device__ __forceinline__ void bw_own(const BwArgs &a, int64_t row, int gl, float (&own)[CPL * 4], float (&v)[CPL * 4]) {
 #pragma unroll
     for (int c = 0; c < CPL; ++c) {
         const int q = gl + c * LPR;
-        if (q < nchunks) ld4<CPL>(base, row, pitch, q, own + c * 4);
-        else {
+        if (q < a.nchunks) {
+            ld4<CPL>(a.mode == 0 ? a.Sk : a.Ybar, row, a.stride, q, own + c * 4);
 #pragma unroll
-            for (int e4 = 0; e4 < 4; ++e4) own[c * 4 + e4] = 0.f;
+            for (int e4 = 0; e4 < 4; ++e4)
+                v[c * 4 + e4] = a.mode == 1 ? own[c * 4 + e4] * (a.a_prev ? __ldg(a.a_prev + q * 4 + e4) : 1.f) : 0.f;
+        } else {
+#pragma unroll
+            for (int e4 = 0; e4 < 4; ++e4) { own[c * 4 + e4] = 0.f; v[c * 4 + e4] = 0.f; }
         }
     }
 }
 
+#ifndef AD_BW_MINB
+#define AD_BW_MINB 3          // CTAs per SM (measured: 3 with 8 neighbours in flight beat 4-6 with 2 or 4)
+#endif
 template <int LPR, int CPL>
-__global__ void __launch_bounds__(256) k_bw(BwArgs a) {
+__global__ void __launch_bounds__(256, AD_BW_MINB) k_bw(BwArgs a) {
     constexpr int E = CPL * 4, G = 32 / LPR;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int grp = lane / LPR, gl = lane % LPR;
+    const unsigned gmask = LPR == 32 ? 0xffffffffu : (((1u << LPR) - 1u) << (grp * LPR));
     const int64_t W = (int64_t)gridDim.x * nwarps;
     for (int64_t task = (int64_t)blockIdx.x * nwarps + warp; task < a.n_tasks; task += W) {
-        float acc_a[E], acc_b[E], own[E];
+        float acc_a[E], acc_b[E], own[E], v[E];
 #pragma unroll
         for (int e = 0; e < E; ++e) { acc_a[e] = 0.f; acc_b[e] = 0.f; }
         if (task < a.n_big) {
@@ -211,8 +339,8 @@ __global__ void __launch_bounds__(256) k_bw(BwArgs a) {
             const int32_t c = a.big_chunk[task];
             const int64_t rb = a.rp[row], re = a.rp[row + 1];
             const int64_t p0 = rb + (int64_t)c * kChunk, p1 = min(re, p0 + kChunk);
-            bw_row<LPR, CPL>(a.Sk, row, a.stride, a.nchunks, gl, own);
-            bw_gather<LPR, CPL>(a, p0, p1, grp, G, gl, acc_a, acc_b);
+            bw_own<LPR, CPL>(a, row, gl, own, v);
+            bw_gather<LPR, CPL>(a, row, p0, p1, grp, G, gl, gmask, v, acc_a, acc_b);
             reduce_groups<LPR, E>(acc_a);
             reduce_groups<LPR, E>(acc_b);
             float *part = a.part + task * (int64_t)2 * a.stride;
@@ -256,288 +384,34 @@ __global__ void __launch_bounds__(256) k_bw(BwArgs a) {
                             }
                         }
                     }
-                    bw_finish<LPR, CPL>(a, row, gl, own, sa, sb);
+                    bw_finish<LPR, CPL>(a, row, gl, gmask, v, own, sa, sb);
                 }
                 if (lane == 0) a.big_counter[t0] = 0u;
             }
         } else if (task < a.n_big + a.n_medium) {
             const int64_t row = a.medium_row[task - a.n_big];
-            bw_row<LPR, CPL>(a.Sk, row, a.stride, a.nchunks, gl, own);
-            bw_gather<LPR, CPL>(a, a.rp[row], a.rp[row + 1], grp, G, gl, acc_a, acc_b);
+            bw_own<LPR, CPL>(a, row, gl, own, v);
+            bw_gather<LPR, CPL>(a, row, a.rp[row], a.rp[row + 1], grp, G, gl, gmask, v, acc_a, acc_b);
             reduce_groups<LPR, E>(acc_a);
             reduce_groups<LPR, E>(acc_b);
-            if (grp == 0) bw_finish<LPR, CPL>(a, row, gl, own, acc_a, acc_b);
+            if (grp == 0) bw_finish<LPR, CPL>(a, row, gl, gmask, v, own, acc_a, acc_b);
         } else {
             const int64_t si = (task - a.n_big - a.n_medium) * G + grp;
             if (si < a.n_small_rows) {
                 const int64_t row = a.small_row[si];
-                bw_row<LPR, CPL>(a.Sk, row, a.stride, a.nchunks, gl, own);
-                bw_gather<LPR, CPL>(a, a.rp[row], a.rp[row + 1], 0, 1, gl, acc_a, acc_b);
-                bw_finish<LPR, CPL>(a, row, gl, own, acc_a, acc_b);
+                bw_own<LPR, CPL>(a, row, gl, own, v);
+                bw_gather<LPR, CPL>(a, row, a.rp[row], a.rp[row + 1], 0, 1, gl, gmask, v, acc_a, acc_b);
+                bw_finish<LPR, CPL>(a, row, gl, gmask, v, own, acc_a, acc_b);
             }
         }
-    }
-}
-
-// ---- sweep backward ----------------------------------------------------------
-// Per row: acc = sum_j w_ij U_j over all entries, and for the entries of its
-// upper part the two dots of the edge.  Bound by the gathers: a lower entry
-// fetches the U half of row j (stride floats), an upper one both halves, 1.5
-// strides per entry on average where fetching [U | s] everywhere took 2; the sum of
-// w s_j that this saves is recovered from G (top of the file).  Backward of R-MAT 22,
-// R = 32, k = 30 with the streaming passes below: 214 -> 132 ms.
-#ifndef AD_BW_MINB
-#define AD_BW_MINB 3          // CTAs per SM (R-MAT 22, k = 30: backward 132 ms; 160 with 2, 166 with 4)
-#endif
-constexpr int kBwUB = 4;      // upper entries in flight per lane group (two row chunks each)
-
-// the upper entries t = first, first + gstride, ... < len at q0, for a lane group;
-// all 32 lanes call it.  au = a U_i, as = a s_i; Gp: accumulators of entry 0.
-template <int LPR, int CPL>
-__device__ __forceinline__ void bw_upper(const BwArgs &a, int64_t q0, int len, int first, int gstride, int gl,
-                                         const float (&au)[CPL * 4], const float (&as)[CPL * 4], double *Gp,
-                                         float (&acc)[CPL * 4]) {
-    constexpr int UB = kBwUB, K = 2 * UB, NC = LPR < UB ? UB / LPR : 1;
-    constexpr int NH = K / LPR > 0 ? K / LPR : 1;
-    constexpr int WS = LPR > K ? LPR / K : 1;   // lanes that hold the same sum
-    const int pitch = 2 * a.stride;
-    int which = 0;                              // first of the sums this lane holds after group_sums
-#pragma unroll
-    for (int o = LPR / 2, c = K; o >= 1; o >>= 1)
-        if (c > 1) {
-            if (gl & o) which += c / 2;
-            c >>= 1;
-        }
-    const bool writer = gl % WS == 0;
-    const int maxlen = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(len - first, 0));
-    int32_t cjn[NC];
-    float wjn[NC];
-    auto load_cols = [&](int b) {
-#pragma unroll
-        for (int i = 0; i < NC; ++i) {
-            const int l = i * LPR + gl, t = first + (b + l) * gstride;
-            const bool ok = l < UB && t < len;
-            cjn[i] = ok ? ld_stream(a.col + q0 + t) : 0;
-            wjn[i] = ok ? (a.w ? ld_stream(a.w + q0 + t) : 1.f) : 0.f;
-        }
-    };
-    load_cols(0);
-    for (int b = 0; b * gstride < maxlen; b += UB) {
-        int32_t cj[NC];
-        float wj[NC];
-#pragma unroll
-        for (int i = 0; i < NC; ++i) { cj[i] = cjn[i]; wj[i] = wjn[i]; }
-        load_cols(b + UB);
-        double gold[NH];   // the accumulators this lane will add to, loaded with the rows
-#pragma unroll
-        for (int i = 0; i < NH; ++i) {
-            const int t = first + (b + (which + i) / 2) * gstride;
-            gold[i] = writer && t < len ? __ldcg(Gp + 2 * (int64_t)t + (which + i) % 2) : 0.0;
-        }
-        float4 uu[UB][CPL], ss[UB][CPL];
-        float wt[UB];
-#pragma unroll
-        for (int u = 0; u < UB; ++u) {
-            const int32_t j = __shfl_sync(0xffffffffu, cj[u / LPR], u % LPR, LPR);
-            wt[u] = __shfl_sync(0xffffffffu, wj[u / LPR], u % LPR, LPR);
-            const bool in = first + (b + u) * gstride < len;
-            const float4 *z = reinterpret_cast<const float4 *>(a.Z + (int64_t)j * pitch);
-#pragma unroll
-            for (int c = 0; c < CPL; ++c) {
-                const int q = gl + c * LPR;
-                const bool ok = in && q < a.nchunks;
-                uu[u][c] = ok ? __ldg(z + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-                ss[u][c] = ok ? __ldg(z + a.stride / 4 + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-        }
-        float dot[K];
-#pragma unroll
-        for (int u = 0; u < UB; ++u) {
-            dot[2 * u] = 0.f;
-            dot[2 * u + 1] = 0.f;
-#pragma unroll
-            for (int c = 0; c < CPL; ++c) {
-                const float uf[4] = {uu[u][c].x, uu[u][c].y, uu[u][c].z, uu[u][c].w};
-                const float sf[4] = {ss[u][c].x, ss[u][c].y, ss[u][c].z, ss[u][c].w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    acc[c * 4 + e] = fmaf(wt[u], uf[e], acc[c * 4 + e]);
-                    dot[2 * u] = fmaf(au[c * 4 + e], sf[e], dot[2 * u]);
-                    dot[2 * u + 1] = fmaf(as[c * 4 + e], uf[e], dot[2 * u + 1]);
-                }
-            }
-        }
-        int w2 = 0;
-        group_sums<LPR, K>(dot, gl, 0xffffffffu, w2);
-#pragma unroll
-        for (int i = 0; i < NH; ++i) {
-            const int t = first + (b + (which + i) / 2) * gstride;
-            if (writer && t < len) Gp[2 * (int64_t)t + (which + i) % 2] = gold[i] + (double)dot[i];
-        }
-    }
-}
-
-// The part [p0, p0 + len) of a row whose upper entries start at `upos`, by the
-// whole warp (WARP) or by a lane group per row; S: sum of w U_j (WARP: over all groups).
-template <int LPR, int CPL, bool WARP>
-__device__ __forceinline__ void bw_part(const BwArgs &a, const SweepArgs &ga, int64_t row, int64_t p0, int len, int lane,
-                                        float (&S)[CPL * 4]) {
-    constexpr int E = CPL * 4, G = 32 / LPR;
-    const int gl = lane % LPR, grp = lane / LPR;
-    const int64_t up = len > 0 ? a.upos[row] : 0;
-    const int lower = len > 0 ? (int)min((int64_t)len, max((int64_t)0, up - p0)) : 0;
-    team_gather<float, LPR, CPL, WARP ? G : 1, 1, AD_SWEEP_UB, false>(ga, p0, lower, lane, S);
-    float au[E], as[E], acc[E];
-    bw_row<LPR, CPL>(a.Z, row, 2 * a.stride, a.nchunks, gl, au);
-    bw_row<LPR, CPL>(a.Z + a.stride, row, 2 * a.stride, a.nchunks, gl, as);
-#pragma unroll
-    for (int c = 0; c < CPL; ++c)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int r = (gl + c * LPR) * 4 + e;
-            const float av = r < a.R ? (a.a_prev ? __ldg(a.a_prev + r) : 1.f) : 0.f;
-            au[c * 4 + e] *= av;
-            as[c * 4 + e] *= av;
-            acc[c * 4 + e] = 0.f;
-        }
-    const int64_t q0 = p0 + lower;
-    double *Gp = a.G + 2 * (len > lower ? a.eoff[row] + (q0 - up) : 0);
-    bw_upper<LPR, CPL>(a, q0, len - lower, WARP ? grp : 0, WARP ? G : 1, gl, au, as, Gp, acc);
-    if (WARP) reduce_groups<LPR, E>(acc);
-#pragma unroll
-    for (int e = 0; e < E; ++e) S[e] += acc[e];
-}
-
-// xbar_{t-1,i} = (1 - omega) ybar_i + omega sum_j w_ij U_j
-template <int LPR, int CPL>
-__device__ __forceinline__ void bw_store(const BwArgs &a, int64_t row, int gl, const float (&S)[CPL * 4]) {
-    const float om = a.omega, om1 = 1.f - a.omega;
-    float4 *xo = reinterpret_cast<float4 *>(a.xbar_out + row * (int64_t)a.stride);
-    const float4 *yb = reinterpret_cast<const float4 *>(a.Ybar + row * (int64_t)a.stride);
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) {
-        const int q = gl + c * LPR;
-        if (q < a.nchunks) {
-            const float4 y = __ldg(yb + q);
-            xo[q] = make_float4(fmaf(om1, y.x, om * S[c * 4]), fmaf(om1, y.y, om * S[c * 4 + 1]),
-                                fmaf(om1, y.z, om * S[c * 4 + 2]), fmaf(om1, y.w, om * S[c * 4 + 3]));
-        }
-    }
-}
-
-template <int LPR, int CPL>
-__global__ void __launch_bounds__(256, AD_BW_MINB) k_bw_sweep(BwArgs a) {
-    constexpr int E = CPL * 4, G = 32 / LPR;
-    const int lane = threadIdx.x & 31, grp = lane / LPR, gl = lane % LPR;
-    SweepArgs ga;                       // what team_gather reads: U_j is the first half of row j of Z
-    ga.col = a.col;
-    ga.w = a.w;
-    ga.x_in = a.Z;
-    ga.stride = 2 * a.stride;
-    ga.nchunks = a.nchunks;
-    const uint32_t n_big = (uint32_t)a.n_big, n_wide = (uint32_t)a.n_wide;
-    const uint32_t n_rows = (uint32_t)(a.n_medium - a.n_wide + a.n_small_rows);   // rows of one lane group
-    const TaskIter it = task_iter(n_big + n_wide + (n_rows + G - 1) / G, 0);
-    for (uint32_t task = it.t; task < it.t_end; task += it.step) {
-        float S[E];
-        if (task < n_big) {
-            // ---- a chunk of a high-degree row; the last chunk adds the partial sums in order
-            const int64_t row = a.big_row[task];
-            const int32_t c = a.big_chunk[task];
-            const int64_t rb = a.rp[row], re = a.rp[row + 1];
-            const int64_t p0 = rb + (int64_t)c * kChunk;
-            bw_part<LPR, CPL, true>(a, ga, row, p0, (int)(min(re, p0 + kChunk) - p0), lane, S);
-            float4 *part = reinterpret_cast<float4 *>(a.part + task * (int64_t)a.stride);
-            if (grp == 0) {
-#pragma unroll
-                for (int cc = 0; cc < CPL; ++cc)
-                    if (gl + cc * LPR < a.nchunks)
-                        __stcg(part + gl + cc * LPR, make_float4(S[cc * 4], S[cc * 4 + 1], S[cc * 4 + 2], S[cc * 4 + 3]));
-                __threadfence();
-            }
-            __syncwarp();
-            const uint32_t t0 = task - c;
-            const int32_t nchunk = (int32_t)((re - rb + kChunk - 1) / kChunk);
-            uint32_t old = 0;
-            if (lane == 0) old = atomicAdd(a.big_counter + t0, 1u);
-            old = __shfl_sync(0xffffffffu, old, 0);
-            if (old == (uint32_t)(nchunk - 1)) {
-                __threadfence();
-                SweepArgs pa;
-                pa.part = a.part;
-                pa.stride = a.stride;
-                pa.nchunks = a.nchunks;
-                sum_partials<float, LPR, CPL>(pa, t0, nchunk, grp, gl, S);
-                if (grp == 0) bw_store<LPR, CPL>(a, row, gl, S);
-                if (lane == 0) a.big_counter[t0] = 0u;
-            }
-        } else if (task < n_big + n_wide) {
-            const int64_t row = a.medium_row[task - n_big];
-            const int64_t p0 = a.rp[row];
-            bw_part<LPR, CPL, true>(a, ga, row, p0, (int)(a.rp[row + 1] - p0), lane, S);
-            if (grp == 0) bw_store<LPR, CPL>(a, row, gl, S);
-        } else {
-            // ---- G rows of about the same degree, one per lane group
-            const uint32_t i = (task - n_big - n_wide) * G + grp, med = (uint32_t)a.n_medium - n_wide;
-            const bool have = i < n_rows;
-            const int64_t row = !have ? 0 : i < med ? a.medium_row[n_wide + i] : a.small_row[i - med];
-            const int64_t p0 = have ? a.rp[row] : 0;
-            bw_part<LPR, CPL, false>(a, ga, row, p0, have ? (int)(a.rp[row + 1] - p0) : 0, lane, S);
-            if (have) bw_store<LPR, CPL>(a, row, gl, S);
-        }
-    }
-}
-
-// C_i = D_i^-1 sum_l w_il G_il in FP64: a warp per chunk or row, a lane per
-// low-degree row; chunks leave their sums in partC, added in order by k_bw_c_big.
-__device__ __forceinline__ double bw_entry_g(const double *G, const int64_t *eid, const float *w, int64_t p, bool upper) {
-    return (w ? (double)w[p] : 1.0) * G[2 * eid[p] + (upper ? 0 : 1)];
-}
-__global__ void k_bw_c(BwArgs a, const double *D, double *C, double *partC) {
-    const int lane = threadIdx.x & 31;
-    const int64_t W = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t n_tasks = a.n_big + a.n_medium + (a.n_small_rows + 31) / 32;
-    for (int64_t task = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); task < n_tasks; task += W) {
-        if (task < a.n_big + a.n_medium) {
-            const bool big = task < a.n_big;
-            const int64_t row = big ? a.big_row[task] : a.medium_row[task - a.n_big];
-            const int64_t p0 = a.rp[row] + (big ? (int64_t)a.big_chunk[task] * kChunk : 0);
-            const int64_t p1 = big ? min(a.rp[row + 1], p0 + kChunk) : a.rp[row + 1], up = a.upos[row];
-            double s = 0.0;
-            for (int64_t p = p0 + lane; p < p1; p += 32) s += bw_entry_g(a.G, a.eid, a.w, p, p >= up);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) {
-                if (big) partC[task] = s;
-                else C[row] = s / D[row];
-            }
-        } else {
-            const int64_t i = (task - a.n_big - a.n_medium) * 32 + lane;
-            if (i < a.n_small_rows) {
-                const int64_t row = a.small_row[i], up = a.upos[row];
-                double s = 0.0;
-                for (int64_t p = a.rp[row]; p < a.rp[row + 1]; ++p) s += bw_entry_g(a.G, a.eid, a.w, p, p >= up);
-                C[row] = s / D[row];
-            }
-        }
-    }
-}
-__global__ void k_bw_c_big(BwArgs a, const double *D, double *C, const double *partC) {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < a.n_big; t += (int64_t)gridDim.x * blockDim.x) {
-        if (a.big_chunk[t] != 0) continue;
-        const int64_t row = a.big_row[t];
-        double s = 0.0;
-        for (int64_t u = t; u < a.n_big && a.big_row[u] == row; ++u) s += partC[u];
-        C[row] = s / D[row];
     }
 }
 
 // per-block partial sums of A = sum xbar (x - 1/2) and B = sum xbar (x + 1/2),
 // x = a (s - lo) - 1/2, and the lowest-index argmin / argmax of each vector
-// of the stored iterate (active rows).  A streaming pass over two blocks: a
-// thread takes one 16-byte chunk of every so many rows.  Products in FP32 (FP64
-// runs on a very narrow pipe on this part), each thread's running sums compensated
-// (Kahan), the threads' sums combined in FP64.  B = A + sum xbar.
+// of the stored iterate (active rows).  Products in FP32 (FP64 runs on a very narrow pipe on
+// this part), each thread's running sums compensated (Kahan), the threads'
+// sums combined in FP64.  B = A + sum xbar.
 constexpr int kRedBlocks = 1216;      // 8 per SM: the per-thread sums are latency bound
 __device__ __forceinline__ void kahan_add(float &sum, float &comp, float x) {
     const float y = x - comp;
@@ -546,51 +420,39 @@ __device__ __forceinline__ void kahan_add(float &sum, float &comp, float x) {
     sum = t;
 }
 
-__global__ void __launch_bounds__(256) k_bw_partial(const float *xbar, const float *S, const int64_t *rp, int64_t n,
-                                                    int32_t stride, int32_t R, const uint32_t *mn, const uint32_t *mx,
-                                                    const float *a_t, double *partA, double *partB,
-                                                    unsigned long long *amin, unsigned long long *amax) {
-    __shared__ double sA[4][256], sX[4][256];
-    const int nq = stride / 4, q = threadIdx.x & (nq - 1);   // stride is a power of two, at most 256
-    const int per = blockDim.x / nq, sub = threadIdx.x / nq;
-    float accA[4], cA[4], accX[4], cX[4], lo[4], hi[4], ar[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        accA[e] = cA[e] = accX[e] = cX[e] = 0.f;
-        const int r = 4 * q + e;
-        lo[e] = r < R ? ord2f(mn[r]) : 0.f;
-        hi[e] = r < R ? ord2f(mx[r]) : 0.f;
-        ar[e] = r < R ? a_t[r] : 0.f;
-    }
-    if (4 * q < R)
-        for (int64_t i = (int64_t)blockIdx.x * per + sub; i < n; i += (int64_t)gridDim.x * per) {
+__global__ void k_bw_partial(const float *xbar, const float *S, const int64_t *rp, int64_t n, int32_t stride, int32_t R,
+                             const uint32_t *mn, const uint32_t *mx, const float *a_t, double *partA, double *partB,
+                             unsigned long long *amin, unsigned long long *amax) {
+    __shared__ double sA[256], sB[256];
+    // thread layout: r = threadIdx.x % R, rows strided over the block's R-wide slices
+    const int Rp = R;
+    const int lanes_per = blockDim.x / Rp > 0 ? blockDim.x / Rp : 1;
+    const int r = threadIdx.x % Rp;
+    const int sub = threadIdx.x / Rp;
+    float accA = 0.f, cA = 0.f, accX = 0.f, cX = 0.f;
+    if (sub < lanes_per && threadIdx.x < lanes_per * Rp) {
+        const float lo = ord2f(mn[r]), hi = ord2f(mx[r]);
+        const float ar = a_t[r];
+        for (int64_t i = (int64_t)blockIdx.x * lanes_per + sub; i < n; i += (int64_t)gridDim.x * lanes_per) {
             if (rp[i + 1] == rp[i]) continue;
-            const float4 xb4 = __ldg(reinterpret_cast<const float4 *>(xbar + i * stride) + q);
-            const float4 s4 = __ldg(reinterpret_cast<const float4 *>(S + i * stride) + q);
-            const float xb[4] = {xb4.x, xb4.y, xb4.z, xb4.w}, sv[4] = {s4.x, s4.y, s4.z, s4.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if (4 * q + e >= R) break;
-                // the lowest-index argmin / argmax of the vector (the rescale's sub-gradient points)
-                if (sv[e] == lo[e]) atomicMin(amin + 4 * q + e, (unsigned long long)i);
-                if (sv[e] == hi[e]) atomicMin(amax + 4 * q + e, (unsigned long long)i);
-                const float xv = ar[e] * (sv[e] - lo[e]) - 0.5f;
-                kahan_add(accA[e], cA[e], xb[e] * (xv - 0.5f));
-                kahan_add(accX[e], cX[e], xb[e]);
-            }
+            const float xb = xbar[i * stride + r];
+            const float sv = S[i * stride + r];
+            // the lowest-index argmin / argmax of vector r (the rescale's sub-gradient points)
+            if (sv == lo) atomicMin(amin + r, (unsigned long long)i);
+            if (sv == hi) atomicMin(amax + r, (unsigned long long)i);
+            const float xv = ar * (sv - lo) - 0.5f;
+            kahan_add(accA, cA, xb * (xv - 0.5f));
+            kahan_add(accX, cX, xb);
         }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        sA[e][threadIdx.x] = (double)accA[e] - (double)cA[e];
-        sX[e][threadIdx.x] = (double)accX[e] - (double)cX[e];
     }
+    sA[threadIdx.x] = (double)accA - (double)cA;
+    sB[threadIdx.x] = (double)accX - (double)cX;
     __syncthreads();
-    if (threadIdx.x < R) {
-        const int e = threadIdx.x & 3, qq = threadIdx.x >> 2;
+    if (threadIdx.x < Rp) {
         double tA = 0.0, tX = 0.0;
-        for (int s2 = 0; s2 < per; ++s2) { tA += sA[e][s2 * nq + qq]; tX += sX[e][s2 * nq + qq]; }
-        partA[(int64_t)blockIdx.x * R + threadIdx.x] = tA;
-        partB[(int64_t)blockIdx.x * R + threadIdx.x] = tA + tX;
+        for (int s2 = 0; s2 < lanes_per; ++s2) { tA += sA[s2 * Rp + threadIdx.x]; tX += sB[s2 * Rp + threadIdx.x]; }
+        partA[(int64_t)blockIdx.x * Rp + threadIdx.x] = tA;
+        partB[(int64_t)blockIdx.x * Rp + threadIdx.x] = tA + tX;
     }
 }
 
@@ -616,48 +478,36 @@ __global__ void k_bw_reduce(const double *partA, const double *partB, int nblock
 }
 
 // ybar = a xbar (+ a A at the argmin, - a B at the argmax); U = D^-1 ybar, written
-// with a copy of s_{t-1} into the rows of Z (the adjoint gather reads both).  A
-// streaming pass, one 16-byte chunk per thread; rows of degree 0 are never read
-// by anything and are left out.  a * xbar in FP32 is the correctly rounded
-// product, i.e. what FP64 then rounding gives; FP64 only at the two corrected
-// entries of each vector.
-__global__ void __launch_bounds__(256) k_bw_ybar(const float *xbar, const int64_t *rp, const float *Dinv, int64_t n,
-                                                 int32_t qshift, int32_t R, const float *a_t, const double *A,
-                                                 const double *B, const unsigned long long *amin,
-                                                 const unsigned long long *amax, float *ybar, const float *S, float *Z) {
-    const int64_t total = n << qshift;
-    const int nq = 1 << qshift;
+// with a copy of s_{t-1} into the rows of Z (the adjoint gather reads both).
+// a * xbar in FP32 is the correctly rounded product, i.e. what FP64 then
+// rounding gives; FP64 only at the two corrected entries of each vector.
+__global__ void k_bw_ybar(const float *xbar, const int64_t *rp, const float *Dinv, int64_t n, int32_t sshift, int32_t R,
+                          const float *a_t, const double *A, const double *B, const unsigned long long *amin,
+                          const unsigned long long *amax, float *ybar, const float *S, float *Z) {
+    const int64_t total = n << sshift;
+    const int rmask = (1 << sshift) - 1;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = t >> qshift;
-        const int q = (int)(t & (nq - 1));
-        if (4 * q >= R || rp[i + 1] == rp[i]) continue;
-        const float4 xb4 = __ldg(reinterpret_cast<const float4 *>(xbar) + t);
-        const float4 s4 = __ldg(reinterpret_cast<const float4 *>(S) + t);
-        const float dinv = __ldg(Dinv + i);
-        const float xb[4] = {xb4.x, xb4.y, xb4.z, xb4.w};
-        float yb[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int r = 4 * q + e;
-            yb[e] = 0.f;
-            if (r < R) {
-                const float ar = __ldg(a_t + r);
-                if (ar > 0.f) {
-                    yb[e] = ar * xb[e];
-                    const bool lo_i = (unsigned long long)i == __ldg(amin + r), hi_i = (unsigned long long)i == __ldg(amax + r);
-                    if (lo_i || hi_i) {
-                        double v = (double)ar * xb[e];
-                        if (lo_i) v += (double)ar * A[r];
-                        if (hi_i) v -= (double)ar * B[r];
-                        yb[e] = (float)v;
-                    }
+        const int64_t i = t >> sshift;
+        const int r = (int)(t & rmask);
+        float yb = 0.f;
+        if (r < R && rp[i + 1] > rp[i]) {
+            const float ar = __ldg(a_t + r);
+            if (ar > 0.f) {
+                const bool lo_i = (unsigned long long)i == amin[r], hi_i = (unsigned long long)i == amax[r];
+                if (lo_i || hi_i) {
+                    double v = (double)ar * xbar[t];
+                    if (lo_i) v += (double)ar * A[r];
+                    if (hi_i) v -= (double)ar * B[r];
+                    yb = (float)v;
+                } else {
+                    yb = ar * xbar[t];
                 }
             }
         }
-        reinterpret_cast<float4 *>(ybar)[t] = make_float4(yb[0], yb[1], yb[2], yb[3]);
-        float4 *z = reinterpret_cast<float4 *>(Z) + (i << (qshift + 1)) + q;   // U and s_{t-1} side by side
-        z[0] = make_float4(yb[0] * dinv, yb[1] * dinv, yb[2] * dinv, yb[3] * dinv);
-        z[nq] = s4;
+        ybar[t] = yb;
+        const int64_t z = (i << (sshift + 1)) + r;   // U and s_{t-1} side by side, twice the pitch
+        Z[z] = yb * Dinv[i];
+        Z[z + (1 << sshift)] = S[t];
     }
 }
 
@@ -668,39 +518,41 @@ __global__ void k_scale_from_mm(const uint32_t *mn, const uint32_t *mx, int32_t 
     a[r] = hi > lo ? 1.f / (hi - lo) : 0.f;
 }
 
-// dL/dw_e = omega (G_p - C_i + G_q - C_j); a thread per CSR entry, the upper ones write
-__global__ void k_edge_grad(const int32_t *col, const int32_t *erow, const int64_t *upos, const int64_t *eoff, int64_t nnz,
-                            const double *G, const double *C, double omega, float *wbar) {
+// dL/dw_e from the per-entry and per-row accumulators of both directions of e
+__global__ void k_edge_grad(const int64_t *rp, const int32_t *col, const int64_t *upos, const int64_t *eoff,
+                            const int64_t *mirror, const int32_t *erow, const double *D, int64_t nnz, const double *G,
+                            const double *C, double omega, float *wbar) {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x) {
         const int32_t i = erow[p], j = col[p];
         if (j <= i) continue;
+        const int64_t q = mirror[p];
         const int64_t e = eoff[i] + (p - upos[i]);
-        wbar[e] = (float)(omega * ((G[2 * e] - C[i]) + (G[2 * e + 1] - C[j])));
+        const double gi = omega * (G[p] - C[i]) / D[i];
+        const double gj = q >= 0 ? omega * (G[q] - C[j]) / D[j] : 0.0;
+        wbar[e] = (float)(gi + gj);
     }
 }
 
 template <int LPR, int CPL>
-static ad_status launch_bw(ad_graph_t g, const BwArgs &a, bool sweep) {
+static ad_status launch_bw(ad_graph_t g, const BwArgs &a) {
     int per_sm = 0;
-    if (sweep) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bw_sweep<LPR, CPL>, 256, 0);
-    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bw<LPR, CPL>, 256, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bw<LPR, CPL>, 256, 0);
     int64_t blocks = (int64_t)(per_sm > 0 ? per_sm : 1) * g->num_sms;
     const int64_t need = (a.n_tasks + 7) / 8;
     if (blocks > need) blocks = need > 0 ? need : 1;
-    if (sweep) AD_LAUNCH((k_bw_sweep<LPR, CPL>), (int)blocks, 256, 0, g->stream, a);
-    else AD_LAUNCH((k_bw<LPR, CPL>), (int)blocks, 256, 0, g->stream, a);
+    AD_LAUNCH((k_bw<LPR, CPL>), (int)blocks, 256, 0, g->stream, a);
     return AD_OK;
 }
 
-static ad_status dispatch_bw(ad_graph_t g, int lpr, int cpl, const BwArgs &a, bool sweep) {
+static ad_status dispatch_bw(ad_graph_t g, int lpr, int cpl, const BwArgs &a) {
     switch (lpr * 100 + cpl) {
-        case 101: return launch_bw<1, 1>(g, a, sweep);
-        case 201: return launch_bw<2, 1>(g, a, sweep);
-        case 401: return launch_bw<4, 1>(g, a, sweep);
-        case 801: return launch_bw<8, 1>(g, a, sweep);
-        case 1601: return launch_bw<16, 1>(g, a, sweep);
-        case 3201: return launch_bw<32, 1>(g, a, sweep);
-        case 3202: return launch_bw<32, 2>(g, a, sweep);
+        case 101: return launch_bw<1, 1>(g, a);
+        case 201: return launch_bw<2, 1>(g, a);
+        case 401: return launch_bw<4, 1>(g, a);
+        case 801: return launch_bw<8, 1>(g, a);
+        case 1601: return launch_bw<16, 1>(g, a);
+        case 3201: return launch_bw<32, 1>(g, a);
+        case 3202: return launch_bw<32, 2>(g, a);
         default: return fail(AD_ERR_INVALID_ARG, "unsupported R for the reverse mode");
     }
 }
@@ -709,7 +561,6 @@ static void fill_bw_plan(BwArgs &a, const RowPlan &p) {
     a.big_row = p.big_row; a.big_chunk = p.big_chunk; a.medium_row = p.medium_row; a.small_row = p.small_row;
     a.big_counter = p.big_counter;
     a.n_big = p.n_big; a.n_medium = p.n_medium; a.n_small_rows = p.n_small_rows;
-    a.n_wide = p.n_wide;
     a.n_tasks = p.tasks();
 }
 
@@ -726,7 +577,7 @@ ad_status backward(ad_graph_t g, const float *rhobar_dev, float *wbar_dev) {
         for (int u = 1; u <= c; ++u) AD_TRY(dalloc_t(g, (n + 1) * stride, &seg[u]));
     float *xbar = nullptr, *xbar2 = nullptr, *ybar = nullptr, *part = nullptr;
     float *a_t = nullptr, *a_p = nullptr, *a_k = nullptr;   // scales of sweep t, t - 1 and k
-    double *G = nullptr, *C = nullptr, *partC = nullptr, *partA = nullptr, *partB = nullptr, *A = nullptr, *B = nullptr;
+    double *G = nullptr, *C = nullptr, *partA = nullptr, *partB = nullptr, *A = nullptr, *B = nullptr;
     unsigned long long *amin = nullptr, *amax = nullptr;
     uint32_t *scratch_mm = nullptr;
     AD_TRY(dalloc_t(g, (n + 1) * stride, &xbar));
@@ -737,9 +588,8 @@ ad_status backward(ad_graph_t g, const float *rhobar_dev, float *wbar_dev) {
     float *Z = nullptr;
     AD_TRY(dalloc_t(g, (n + 1) * 2 * (size_t)stride, &Z));
     AD_TRY(dalloc_t(g, (size_t)std::max<int64_t>(plan->n_big, 1) * 2 * stride, &part));
-    AD_TRY(dalloc_t(g, 2 * (size_t)g->m + 2, &G));
+    AD_TRY(dalloc_t(g, nnz + 1, &G));
     AD_TRY(dalloc_t(g, n + 1, &C));
-    AD_TRY(dalloc_t(g, (size_t)std::max<int64_t>(plan->n_big, 1), &partC));
     AD_TRY(dalloc_t(g, (size_t)kRedBlocks * stride, &partA));
     AD_TRY(dalloc_t(g, (size_t)kRedBlocks * stride, &partB));
     AD_TRY(dalloc_t(g, stride, &A));
@@ -750,10 +600,11 @@ ad_status backward(ad_graph_t g, const float *rhobar_dev, float *wbar_dev) {
     AD_TRY(dalloc_t(g, stride, &a_p));
     AD_TRY(dalloc_t(g, stride, &a_k));
     AD_TRY(dalloc_t(g, 2 * stride, &scratch_mm));
-    AD_CUDA_TRY(cudaMemsetAsync(G, 0, 2 * (size_t)g->m * sizeof(double), g->stream));
+    AD_CUDA_TRY(cudaMemsetAsync(G, 0, (nnz + 1) * sizeof(double), g->stream));
+    AD_CUDA_TRY(cudaMemsetAsync(C, 0, (n + 1) * sizeof(double), g->stream));
     const uint32_t *mm_min = sv->mm, *mm_max = sv->mm + (size_t)k * stride;
-    int qshift = 0;   // stride / 4 = 1 << qshift (a power of two)
-    while ((4 << qshift) < stride) ++qshift;
+    int sshift = 0;   // stride = 1 << sshift (a power of two, at least 4)
+    while ((1 << sshift) < stride) ++sshift;
     auto slot_min = [&](int t) { return mm_min + (size_t)(t - 1) * stride; };   // min/max of s_t, t >= 1
     auto slot_max = [&](int t) { return mm_max + (size_t)(t - 1) * stride; };
 
@@ -762,8 +613,7 @@ ad_status backward(ad_graph_t g, const float *rhobar_dev, float *wbar_dev) {
     a.rp = g->rp; a.col = g->col; a.w = g->w; a.Dinv = g->Dinv; a.eid = g->eid;
     a.stride = stride; a.nchunks = sv->nchunks; a.R = R; a.omega = (float)sv->omega;
     a.rho = sv->rho; a.rhobar = rhobar_dev;
-    a.upos = g->upos; a.eoff = g->eoff;
-    a.G = G; a.part = part;
+    a.G = G; a.C = C; a.part = part;
     fill_bw_plan(a, *plan);
 
     const int nseg = k > 0 ? (k + c - 1) / c : 0;
@@ -790,9 +640,10 @@ ad_status backward(ad_graph_t g, const float *rhobar_dev, float *wbar_dev) {
         if (!have_xbar) {   // distance backward on s_k
             AD_LAUNCH(k_scale_from_mm, 1, 256, 0, g->stream, slot_min(k), slot_max(k), stride, a_k);
             a.a_k = a_k;
+            a.mode = 0;
             a.Sk = seg[len];
             a.xbar_out = xbar;
-            AD_TRY(dispatch_bw(g, sv->lpr, sv->cpl, a, false));
+            AD_TRY(dispatch_bw(g, sv->lpr, sv->cpl, a));
             have_xbar = true;
         }
         for (int u = len; u >= 1; --u) {
@@ -805,7 +656,7 @@ ad_status backward(ad_graph_t g, const float *rhobar_dev, float *wbar_dev) {
             AD_LAUNCH(k_bw_partial, kRedBlocks, 256, 0, g->stream, xbar, St, g->rp, n, stride, R, slot_min(t),
                       slot_max(t), a_t, partA, partB, amin, amax);
             AD_LAUNCH(k_bw_reduce, 1, 1024, 0, g->stream, partA, partB, kRedBlocks, R, A, B);
-            AD_LAUNCH(k_bw_ybar, g->num_sms * 16, 256, 0, g->stream, xbar, g->rp, g->Dinv, n, qshift, R, a_t, A, B, amin,
+            AD_LAUNCH(k_bw_ybar, g->num_sms * 16, 256, 0, g->stream, xbar, g->rp, g->Dinv, n, sshift, R, a_t, A, B, amin,
                       amax, ybar, Sp, Z);
             // sweep adjoint + weight terms
             if (t >= 2) {
@@ -814,21 +665,22 @@ ad_status backward(ad_graph_t g, const float *rhobar_dev, float *wbar_dev) {
             } else {
                 a.a_prev = nullptr;
             }
-            a.Z = Z;
+            a.mode = 1;
+            a.U = Z;
+            a.Sprev = Z + stride;
+            a.gpitch = 2 * stride;
             a.Ybar = ybar;
             a.xbar_out = xbar2;
-            AD_TRY(dispatch_bw(g, sv->lpr, sv->cpl, a, true));
+            AD_TRY(dispatch_bw(g, sv->lpr, sv->cpl, a));
             std::swap(xbar, xbar2);
         }
     }
-    AD_LAUNCH(k_bw_c, g->num_sms * 8, 256, 0, g->stream, a, g->D, C, partC);
-    if (a.n_big > 0) AD_LAUNCH(k_bw_c_big, g->num_sms, 256, 0, g->stream, a, g->D, C, partC);
-    AD_LAUNCH(k_edge_grad, g->num_sms * 16, 256, 0, g->stream, g->col, g->erow, g->upos, g->eoff, nnz, G, C, sv->omega,
-              wbar_dev);
+    AD_LAUNCH(k_edge_grad, g->num_sms * 16, 256, 0, g->stream, g->rp, g->col, g->upos, g->eoff, g->mirror, g->erow, g->D,
+              nnz, G, C, sv->omega, wbar_dev);
     AD_CUDA_TRY(cudaStreamSynchronize(g->stream));
     if (!sv->all)
         for (int u = 1; u <= c; ++u) dfree(g, seg[u]);
-    for (void *p : {(void *)xbar, (void *)xbar2, (void *)ybar, (void *)Z, (void *)part, (void *)G, (void *)C, (void *)partC,
+    for (void *p : {(void *)xbar, (void *)xbar2, (void *)ybar, (void *)Z, (void *)part, (void *)G, (void *)C,
                     (void *)partA, (void *)partB, (void *)A, (void *)B, (void *)amin, (void *)amax, (void *)a_t, (void *)a_p, (void *)a_k,
                     (void *)scratch_mm})
         dfree(g, p);

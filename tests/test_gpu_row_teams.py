@@ -61,15 +61,3 @@ def test_batch_equals_its_graphs(R, storage):
         h = L.ad_graph_create(g.n, g.row_ptr, g.col, None)
         assert np.array_equal(rho[at[k]:at[k + 1]], distances(L, h, g.m, R, storage)), k
         L.ad_graph_destroy(h)
-
-
-@pytest.mark.parametrize("weighted", [False, True])
-@pytest.mark.parametrize("R", [2, 7, 16, 32, 64, 130])
-def test_gradient_at_degree_borders(R, weighted):
-    # every row class with its lower and upper parts; the bound of test_gpu_grad.py
-    from test_gpu_grad import GRAD_TOL, gpu_loss_grad, grad_error
-    g = border_graph(weighted, copies=2)
-    S = graphgen.random_edge_subset(g.m, 0.2, seed=3)
-    _, wb = gpu_loss_grad(g, S, R, 4, 0.5, 11)
-    _, ref = oracle.loss_grad(g.row_ptr, g.col, entry_weights_f64(g), S, R=R, k=4, omega=0.5, seed=11)
-    assert grad_error(wb, ref) <= GRAD_TOL
