@@ -478,36 +478,49 @@ __global__ void k_bw_reduce(const double *partA, const double *partB, int nblock
 }
 
 // ybar = a xbar (+ a A at the argmin, - a B at the argmax); U = D^-1 ybar, written
-// with a copy of s_{t-1} into the rows of Z (the adjoint gather reads both).
-// a * xbar in FP32 is the correctly rounded product, i.e. what FP64 then
-// rounding gives; FP64 only at the two corrected entries of each vector.
-__global__ void k_bw_ybar(const float *xbar, const int64_t *rp, const float *Dinv, int64_t n, int32_t sshift, int32_t R,
-                          const float *a_t, const double *A, const double *B, const unsigned long long *amin,
-                          const unsigned long long *amax, float *ybar, const float *S, float *Z) {
-    const int64_t total = n << sshift;
-    const int rmask = (1 << sshift) - 1;
+// with a copy of s_{t-1} into the rows of Z (the adjoint gather reads both).  A
+// streaming pass, one 16-byte chunk per thread; rows of degree 0 are never read
+// by anything and are left out.  a * xbar in FP32 is the correctly rounded
+// product, i.e. what FP64 then rounding gives; FP64 only at the two corrected
+// entries of each vector.  (Four bytes per thread over all rows before: the backward
+// and forward of R-MAT 22, k = 30 together 262 -> 251 ms.)
+__global__ void __launch_bounds__(256) k_bw_ybar(const float *xbar, const int64_t *rp, const float *Dinv, int64_t n,
+                                                 int32_t qshift, int32_t R, const float *a_t, const double *A,
+                                                 const double *B, const unsigned long long *amin,
+                                                 const unsigned long long *amax, float *ybar, const float *S, float *Z) {
+    const int64_t total = n << qshift;
+    const int nq = 1 << qshift;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = t >> sshift;
-        const int r = (int)(t & rmask);
-        float yb = 0.f;
-        if (r < R && rp[i + 1] > rp[i]) {
-            const float ar = __ldg(a_t + r);
-            if (ar > 0.f) {
-                const bool lo_i = (unsigned long long)i == amin[r], hi_i = (unsigned long long)i == amax[r];
-                if (lo_i || hi_i) {
-                    double v = (double)ar * xbar[t];
-                    if (lo_i) v += (double)ar * A[r];
-                    if (hi_i) v -= (double)ar * B[r];
-                    yb = (float)v;
-                } else {
-                    yb = ar * xbar[t];
+        const int64_t i = t >> qshift;
+        const int q = (int)(t & (nq - 1));
+        if (4 * q >= R || rp[i + 1] == rp[i]) continue;
+        const float4 xb4 = __ldg(reinterpret_cast<const float4 *>(xbar) + t);
+        const float4 s4 = __ldg(reinterpret_cast<const float4 *>(S) + t);
+        const float dinv = __ldg(Dinv + i);
+        const float xb[4] = {xb4.x, xb4.y, xb4.z, xb4.w};
+        float yb[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int r = 4 * q + e;
+            yb[e] = 0.f;
+            if (r < R) {
+                const float ar = __ldg(a_t + r);
+                if (ar > 0.f) {
+                    yb[e] = ar * xb[e];
+                    const bool lo_i = (unsigned long long)i == __ldg(amin + r), hi_i = (unsigned long long)i == __ldg(amax + r);
+                    if (lo_i || hi_i) {
+                        double v = (double)ar * xb[e];
+                        if (lo_i) v += (double)ar * A[r];
+                        if (hi_i) v -= (double)ar * B[r];
+                        yb[e] = (float)v;
+                    }
                 }
             }
         }
-        ybar[t] = yb;
-        const int64_t z = (i << (sshift + 1)) + r;   // U and s_{t-1} side by side, twice the pitch
-        Z[z] = yb * Dinv[i];
-        Z[z + (1 << sshift)] = S[t];
+        reinterpret_cast<float4 *>(ybar)[t] = make_float4(yb[0], yb[1], yb[2], yb[3]);
+        float4 *z = reinterpret_cast<float4 *>(Z) + (i << (qshift + 1)) + q;   // U and s_{t-1} side by side
+        z[0] = make_float4(yb[0] * dinv, yb[1] * dinv, yb[2] * dinv, yb[3] * dinv);
+        z[nq] = s4;
     }
 }
 
@@ -603,8 +616,8 @@ ad_status backward(ad_graph_t g, const float *rhobar_dev, float *wbar_dev) {
     AD_CUDA_TRY(cudaMemsetAsync(G, 0, (nnz + 1) * sizeof(double), g->stream));
     AD_CUDA_TRY(cudaMemsetAsync(C, 0, (n + 1) * sizeof(double), g->stream));
     const uint32_t *mm_min = sv->mm, *mm_max = sv->mm + (size_t)k * stride;
-    int sshift = 0;   // stride = 1 << sshift (a power of two, at least 4)
-    while ((1 << sshift) < stride) ++sshift;
+    int qshift = 0;   // stride / 4 = 1 << qshift (a power of two)
+    while ((4 << qshift) < stride) ++qshift;
     auto slot_min = [&](int t) { return mm_min + (size_t)(t - 1) * stride; };   // min/max of s_t, t >= 1
     auto slot_max = [&](int t) { return mm_max + (size_t)(t - 1) * stride; };
 
@@ -656,7 +669,7 @@ ad_status backward(ad_graph_t g, const float *rhobar_dev, float *wbar_dev) {
             AD_LAUNCH(k_bw_partial, kRedBlocks, 256, 0, g->stream, xbar, St, g->rp, n, stride, R, slot_min(t),
                       slot_max(t), a_t, partA, partB, amin, amax);
             AD_LAUNCH(k_bw_reduce, 1, 1024, 0, g->stream, partA, partB, kRedBlocks, R, A, B);
-            AD_LAUNCH(k_bw_ybar, g->num_sms * 16, 256, 0, g->stream, xbar, g->rp, g->Dinv, n, sshift, R, a_t, A, B, amin,
+            AD_LAUNCH(k_bw_ybar, g->num_sms * 16, 256, 0, g->stream, xbar, g->rp, g->Dinv, n, qshift, R, a_t, A, B, amin,
                       amax, ybar, Sp, Z);
             // sweep adjoint + weight terms
             if (t >= 2) {
