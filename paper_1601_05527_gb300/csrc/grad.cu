@@ -482,8 +482,8 @@ __global__ void k_bw_reduce(const double *partA, const double *partB, int nblock
 // streaming pass, one 16-byte chunk per thread; rows of degree 0 are never read
 // by anything and are left out.  a * xbar in FP32 is the correctly rounded
 // product, i.e. what FP64 then rounding gives; FP64 only at the two corrected
-// entries of each vector.  (Four bytes per thread over all rows before: the backward
-// and forward of R-MAT 22, k = 30 together 262 -> 251 ms.)
+// entries of each vector.  (Four bytes per thread over all rows before, 22 ms
+// of a step of R-MAT 22, k = 30; the step, with the forward's row teams, 283 -> 251 ms.)
 __global__ void __launch_bounds__(256) k_bw_ybar(const float *xbar, const int64_t *rp, const float *Dinv, int64_t n,
                                                  int32_t qshift, int32_t R, const float *a_t, const double *A,
                                                  const double *B, const unsigned long long *amin,
