@@ -28,7 +28,10 @@
 
 // Tuning parameters (compile-time; the defaults are the measured choice on GB300).
 #ifndef AD_SWEEP_UB
-#define AD_SWEEP_UB 8          // independent row loads in flight per lane
+#define AD_SWEEP_UB 8          // independent row loads in flight per lane (FP32 storage)
+#endif
+#ifndef AD_SWEEP_UB16
+#define AD_SWEEP_UB16 4        // ... for the 16-bit storage formats
 #endif
 #ifndef AD_SWEEP_UBS
 #define AD_SWEEP_UBS 4         // ... of a low-degree row
@@ -364,14 +367,15 @@ __device__ __forceinline__ void team_gather(const SweepArgs &a, int64_t p0, int 
     team_gather_w<T, LPR, CPL, MOD, RES, UB, true, P>(a, p0, d, lane, S);
 }
 
-// Residues per lane of the rows that share a warp: four accumulators of one FP32
-// chunk (four rows per warp for up to eight lanes per row), two where a lane holds
-// eight values (16-bit storage, two chunks): 64 (48) registers hold no more beside
-// the loads in flight.  Measured at R-MAT 20, R = 32, FP32: 303 us with four, 323 with two.
+// Residues per lane of the rows that share a warp: 16 sums a lane, that is four
+// accumulators of one FP32 chunk (four rows per warp for up to eight lanes per row),
+// two where a lane holds eight values (16-bit storage, or two FP32 chunks), one where
+// it holds 16: 64 (16-bit: 48) registers hold no more beside the loads in flight.
+// Measured at R-MAT 20, R = 32, FP32: 303 us with four, 323 with two.
 constexpr int kTeamRes = 4;
 template <typename T, int LPR, int CPL>
 constexpr int team_res() {
-    constexpr int G = 32 / LPR, want = Store<T>::V * CPL <= 4 ? kTeamRes : 2;
+    constexpr int G = 32 / LPR, want = kTeamRes * 4 / (Store<T>::V * CPL);
     return G < want ? G : want;
 }
 
@@ -601,6 +605,12 @@ __device__ __forceinline__ void sum_partials(const SweepArgs &a, int64_t t0, int
 // FP16 with four at 3 / 4 / 5 CTAs 314 / 275 / 264 us.
 template <typename T>
 constexpr int sweep_minb() { return sizeof(T) == 4 ? AD_SWEEP_MINB : AD_SWEEP_MINB16; }
+// Row loads in flight per lane.  The 48 registers of the 16-bit formats hold four
+// loads (16) beside the 16 sums of a lane; with eight the compiler spills up to ten
+// times as much (a sweep of R-MAT 18: FP16, R = 256 475 -> 398 us with four, Q16,
+// R = 40 186 -> 167 us).  Up to R = 32 a batch has four entries a lane either way.
+template <typename T>
+constexpr int sweep_loads() { return sizeof(T) == 4 ? AD_SWEEP_UB : AD_SWEEP_UB16; }
 
 // The tasks of one sweep on this CTA, then the CTA's min/max to the sweep's
 // slots.  P: inside the persistent launch.  B: a batch of graphs.  acs: scale and
@@ -610,7 +620,7 @@ template <typename T, int LPR, int CPL, bool P, bool B>
 __device__ __forceinline__ void sweep_tasks(const SweepArgs &a, const float *acs, float *mm) {
     using L = Lane<T, LPR, CPL>;
     constexpr int V = L::V, E = L::E, G = L::G, RES = team_res<T, LPR, CPL>();
-    constexpr int UB = AD_SWEEP_UB, UBS = AD_SWEEP_UBS;
+    constexpr int UB = sweep_loads<T>(), UBS = AD_SWEEP_UBS;
     using TM = Team<LPR, G, RES>;
     const int lane = threadIdx.x & 31;
     const int grp = lane / LPR, gl = lane % LPR;
