@@ -264,6 +264,8 @@ struct ad_graph_s {
     double *D = nullptr;         // weighted degree (FP64)
     uint8_t *dexact = nullptr;   // [n] weighted graphs: 1 where every partial sum of the row's weights is exact in FP64
     float *Dinv = nullptr;       // 1 / D (0 for isolated vertices)
+    int64_t n_long_rows = 0;     // rows summed by a block each (graph.cu)
+    int32_t *long_rows = nullptr;   // [n_long_rows] (weighted graphs)
     int64_t *upos = nullptr;     // first CSR position of row i with col > i
     int64_t *eoff = nullptr;     // edge id of that position; eoff[n] = m
     int64_t *mirror = nullptr;   // [nnz] position of the reverse entry (built lazily)

@@ -236,9 +236,9 @@ __global__ void k_degrees(const int64_t *rp, const int32_t *col, const float *w,
 // lane.  exact_out[i] records which case row i is (the seed rule relies on it).
 __device__ __forceinline__ int fp32_biased_exponent(float v) { return (int)((__float_as_uint(v) >> 23) & 0xffu); }
 
-// Rows longer than kLongDegreeRow are only listed (long_rows[0 .. *n_long)): one
-// warp would hold the launch up on a hub for milliseconds (R-MAT 22: 4.9 ms, all of
-// it hubs); k_wdegrees_long gives each a block.
+// Rows longer than kLongDegreeRow are left out: one warp would hold the launch up on
+// a hub for milliseconds (R-MAT 22: 4.9 ms, all of it hubs); k_wdegrees_long gives
+// each a block.
 constexpr int64_t kLongDegreeRow = 2048;
 __device__ __forceinline__ bool sum_is_exact(int64_t d, int emax, int emin) {
     int lg = 0;
@@ -247,16 +247,12 @@ __device__ __forceinline__ bool sum_is_exact(int64_t d, int emax, int emin) {
     return d == 0 || emax - max(emin, 1) + lg + 24 <= 53;
 }
 
-__global__ void k_wdegrees(const int64_t *rp, const float *w, int64_t n, double *D, float *Dinv, uint8_t *exact_out,
-                           int32_t *long_rows, unsigned int *n_long) {
+__global__ void k_wdegrees(const int64_t *rp, const float *w, int64_t n, double *D, float *Dinv, uint8_t *exact_out) {
     const int lane = threadIdx.x & 31;
     const int64_t W = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += W) {
         const int64_t b = rp[i], e = rp[i + 1];
-        if (e - b > kLongDegreeRow) {
-            if (lane == 0) long_rows[atomicAdd(n_long, 1u)] = (int32_t)i;
-            continue;
-        }
+        if (e - b > kLongDegreeRow) continue;
         double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;   // four independent loads in flight per lane
         int emax = 0, emin = 255;
         int64_t p = b + lane;
@@ -297,19 +293,25 @@ __global__ void k_wdegrees(const int64_t *rp, const float *w, int64_t n, double 
     }
 }
 
-// The listed long rows, a block each: the same sum where it is exact, otherwise
+// The rows of more than kLongDegreeRow entries, in any order: they do not change with
+// the weights, so the list is made once per handle.
+__global__ void k_list_long_rows(const int64_t *rp, int64_t n, int32_t *rows, unsigned int *count) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        if (rp[i + 1] - rp[i] > kLongDegreeRow) rows[atomicAdd(count, 1u)] = (int32_t)i;
+}
+
+// The long rows, a block each: the same sum where it is exact, otherwise
 // one after the other in CSR order by one thread, from shared memory.
 constexpr int kLongDegreeThreads = 512;
 __global__ void __launch_bounds__(kLongDegreeThreads) k_wdegrees_long(const int64_t *rp, const float *w,
-                                                                      const int32_t *rows, const unsigned int *n_rows,
-                                                                      double *D, float *Dinv, uint8_t *exact_out) {
+                                                                      const int32_t *rows, int64_t count, double *D,
+                                                                      float *Dinv, uint8_t *exact_out) {
     constexpr int T = kLongDegreeThreads, NW = T / 32, kTile = 4 * T;
     __shared__ double ssum[NW];
     __shared__ int smax[NW], smin[NW];
     __shared__ float tile[kTile];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned int count = *n_rows;
-    for (unsigned int t = blockIdx.x; t < count; t += gridDim.x) {
+    for (int64_t t = blockIdx.x; t < count; t += gridDim.x) {
         const int64_t i = rows[t], b = rp[i], e = rp[i + 1];
         double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
         int emax = 0, emin = 255;
@@ -473,18 +475,20 @@ ad_status recompute_degrees(ad_graph_t g) {
     const int64_t tblocks = std::min<int64_t>((g->n + 255) / 256 + 1, (int64_t)g->num_sms * 16);
     AD_LAUNCH(k_degrees, (int)tblocks, 256, 0, g->stream, g->rp, g->col, g->w, g->n, g->D, g->Dinv, g->upos,
               ucount);
-    int32_t *lrows = nullptr;
     if (g->w) {
         const int64_t wblocks = std::min<int64_t>((g->n + 7) / 8 + 1, (int64_t)g->num_sms * 64);
         if (!g->dexact) AD_TRY(dalloc_t(g, g->n + 1, &g->dexact));
-        const int64_t cap = g->nnz / kLongDegreeRow + 1;   // more rows cannot be that long
-        AD_TRY(dalloc_t(g, cap + 1, &lrows));
-        unsigned int *n_long = reinterpret_cast<unsigned int *>(lrows + cap);
-        AD_CUDA_TRY(cudaMemsetAsync(n_long, 0, sizeof(unsigned int), g->stream));
-        AD_LAUNCH(k_wdegrees, (int)wblocks, 256, 0, g->stream, g->rp, g->w, g->n, g->D, g->Dinv, g->dexact, lrows, n_long);
-        if (cap > 1)
-            AD_LAUNCH(k_wdegrees_long, (int)std::min<int64_t>(cap, (int64_t)g->num_sms * 4), kLongDegreeThreads, 0,
-                      g->stream, g->rp, g->w, lrows, n_long, g->D, g->Dinv, g->dexact);
+        AD_LAUNCH(k_wdegrees, (int)wblocks, 256, 0, g->stream, g->rp, g->w, g->n, g->D, g->Dinv, g->dexact);
+        if (g->n_long_rows > 0) {
+            if (!g->long_rows) {   // the last slot counts while the list is filled
+                AD_TRY(dalloc_t(g, g->n_long_rows + 1, &g->long_rows));
+                unsigned int *count = reinterpret_cast<unsigned int *>(g->long_rows + g->n_long_rows);
+                AD_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(unsigned int), g->stream));
+                AD_LAUNCH(k_list_long_rows, (int)tblocks, 256, 0, g->stream, g->rp, g->n, g->long_rows, count);
+            }
+            AD_LAUNCH(k_wdegrees_long, (int)std::min<int64_t>(g->n_long_rows, (int64_t)g->num_sms * 4), kLongDegreeThreads,
+                      0, g->stream, g->rp, g->w, g->long_rows, g->n_long_rows, g->D, g->Dinv, g->dexact);
+        }
     }
     int64_t m = 0;
     ad_status st = exclusive_scan_i64(g, ucount, g->eoff, g->n, &m);
@@ -492,18 +496,22 @@ ad_status recompute_degrees(ad_graph_t g) {
     AD_TRY(st);
     AD_CUDA_TRY(cudaMemcpyAsync(g->eoff + g->n, &m, sizeof(int64_t), cudaMemcpyHostToDevice, g->stream));
     AD_CUDA_TRY(cudaStreamSynchronize(g->stream));
-    if (lrows) dfree(g, lrows);
     g->m = m;
     return compute_anchors(g);
 }
 
+// cnt[0]: rows of degree > 0; cnt[1]: rows of more than kLongDegreeRow entries
 __global__ void k_count_active(const int64_t *rp, int64_t n, unsigned long long *cnt) {
-    unsigned long long c = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        c += (rp[i + 1] > rp[i]) ? 1 : 0;
+    unsigned long long c = 0, l = 0;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t d = rp[i + 1] - rp[i];
+        c += d > 0 ? 1 : 0;
+        l += d > kLongDegreeRow ? 1 : 0;
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(cnt, c);
+    if (l) atomicAdd(cnt + 1, l);
 }
 
 // out[k] = src[idx[k]] (idx[k] >= limit: fill); a handful of values read back with one copy
@@ -515,10 +523,10 @@ __global__ void k_pick_i64(const int64_t *src, const int64_t *idx, int64_t count
 
 ad_status graph_setup(ad_graph_t g, int32_t flags) {
     const int64_t n = g->n;
-    unsigned long long *err = nullptr;   // [0] first violation, [1] active rows, [2] pairs found
-    AD_TRY(dalloc_t(g, 3, &err));
+    unsigned long long *err = nullptr;   // [0] first violation, [1] pairs found, [2] active rows, [3] long rows
+    AD_TRY(dalloc_t(g, 4, &err));
     AD_CUDA_TRY(cudaMemsetAsync(err, 0xff, sizeof(unsigned long long), g->stream));
-    AD_CUDA_TRY(cudaMemsetAsync(err + 1, 0, 2 * sizeof(unsigned long long), g->stream));
+    AD_CUDA_TRY(cudaMemsetAsync(err + 1, 0, 3 * sizeof(unsigned long long), g->stream));
     const int grid = g->num_sms * 8;
     if (!(flags & AD_CREATE_SKIP_VALIDATION)) {
         AD_LAUNCH(k_check_rows, grid, 256, 0, g->stream, g->rp, n, g->nnz, err);
@@ -530,10 +538,10 @@ ad_status graph_setup(ad_graph_t g, int32_t flags) {
             const int64_t wblocks = std::min<int64_t>((n + 255) / 256 + 1, (int64_t)g->num_sms * 16);
             AD_LAUNCH(k_entry_rows, (int)wblocks, 256, 0, g->stream, g->rp, n, g->erow);
             AD_LAUNCH(k_check_pairs, g->num_sms * 16, 256, 0, g->stream, g->rp, g->col, g->w, g->erow, n, g->nnz,
-                      g->voff, g->G, err, err + 2, g->mirror);
-            unsigned long long fast[3] = {0, 0, 0};
+                      g->voff, g->G, err, err + 1, g->mirror);
+            unsigned long long fast[2] = {0, 0};
             AD_TRY(copy_out(g, fast, err, sizeof(fast)));
-            if (fast[0] != ~0ull || 2 * fast[2] != (unsigned long long)g->nnz) {
+            if (fast[0] != ~0ull || 2 * fast[1] != (unsigned long long)g->nnz) {
                 // a violation: the per-entry pass reports the first one by priority and position
                 AD_CUDA_TRY(cudaMemsetAsync(err, 0xff, sizeof(unsigned long long), g->stream));
                 AD_LAUNCH(k_check_entries, g->num_sms * 16, 256, 0, g->stream, g->rp, g->col, g->w, g->erow, n,
@@ -549,10 +557,11 @@ ad_status graph_setup(ad_graph_t g, int32_t flags) {
                                              (prio == P_CSR ? "index " : "CSR entry ") + std::to_string(pos));
         }
     }
-    AD_LAUNCH(k_count_active, grid, 256, 0, g->stream, g->rp, n, err + 1);
-    unsigned long long na = 0;
-    AD_TRY(copy_out(g, &na, err + 1, sizeof(na)));
-    g->n_active = (int64_t)na;
+    AD_LAUNCH(k_count_active, grid, 256, 0, g->stream, g->rp, n, err + 2);
+    unsigned long long na[2] = {0, 0};
+    AD_TRY(copy_out(g, na, err + 2, sizeof(na)));
+    g->n_active = (int64_t)na[0];
+    g->n_long_rows = (int64_t)na[1];
     dfree(g, err);
     AD_TRY(dalloc_t(g, n + 1, &g->D));
     AD_TRY(dalloc_t(g, n + 1, &g->Dinv));
