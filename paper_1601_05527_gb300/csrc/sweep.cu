@@ -78,12 +78,19 @@ ad_status get_row_plan(ad_graph_t g, int groups, bool upper, RowPlan **out) {
     return AD_OK;
 }
 
-static void fill_plan(SweepArgs &a, const RowPlan &p) {
+// Where a task for every medium row comes to no more than half of the resident warps,
+// the rows of the sweep do not share warps: a row's chain is shorter alone, and the
+// warps are there (the same sums either way).  Barabasi-Albert 1K, R = 16, k = 20, FP32:
+// 175 -> 123 us a call; 3K, R = 10 180 -> 148 us.  Up to all resident warps it loses as often as it
+// gains: 6K, FP16, R = 48 310 -> 327 us, 64x64 grid, FP32, R = 48 123 -> 138 us.
+constexpr int64_t kSmallTasks = 16;   // tasks per SM
+
+static void fill_plan(ad_graph_t g, SweepArgs &a, const RowPlan &p) {
     a.big_row = p.big_row; a.big_chunk = p.big_chunk; a.medium_row = p.medium_row; a.small_row = p.small_row;
     a.big_counter = p.big_counter;
     a.n_big = p.n_big; a.n_medium = p.n_medium; a.n_small_rows = p.n_small_rows;
-    a.n_wide = p.n_wide;
     a.n_tasks = p.tasks();
+    a.n_wide = a.n_tasks <= kSmallTasks * g->num_sms ? p.n_medium : p.n_wide;
 }
 
 static void ev_begin(ad_graph_t g) {
@@ -118,7 +125,7 @@ ad_status sweep_step(ad_graph_t g, ad_storage storage, int32_t R, double omega, 
     a.anchor = g->anchor;
     AD_TRY(ensure(g, g->ac, (size_t)g->G * 2 * cf.stride * sizeof(float)));
     a.ac = static_cast<float *>(g->ac.ptr);
-    fill_plan(a, *sp);
+    fill_plan(g, a, *sp);
     a.x_in = x_in; a.x_out = x_out;
     a.mm_prev_min = pmin; a.mm_prev_max = pmax; a.mm_min = mn; a.mm_max = mx;
     return dispatch_storage(g, storage, cf, true, a, sweep_smem(cf.stride, g->G > 1));
@@ -157,8 +164,8 @@ static ad_status relax_persistent(ad_graph_t g, const Config &cf, int32_t R, int
     a.voff = g->voff; a.G = 1; a.blocked = 0;
     a.anchor = g->anchor;
     r.d = a;
-    fill_plan(r.s, sp);
-    fill_plan(r.d, dp);
+    fill_plan(g, r.s, sp);
+    fill_plan(g, r.d, dp);
     r.d.rho = rho_dev;
     r.n = g->n;
     r.k = k;
@@ -283,7 +290,7 @@ ad_status algebraic_distance(ad_graph_t g, int32_t R, int32_t k, double omega, u
     const bool direct = keep && keep->every == 1 && keep->ckpt.size() == (size_t)k + 1;
     if (direct) xin = keep->ckpt[0];
     const size_t smem = sweep_smem(cf.stride, g->G > 1);
-    fill_plan(a, *sp);
+    fill_plan(g, a, *sp);
     for (int32_t t = 0; t < k; ++t) {
         if (direct) xout = keep->ckpt[t + 1];
         a.x_in = xin; a.x_out = xout;
@@ -304,7 +311,7 @@ ad_status algebraic_distance(ad_graph_t g, int32_t R, int32_t k, double omega, u
         AD_CUDA_TRY(cudaMemcpyAsync(keep->mm_copy, g->mm.ptr, 2 * mm_words * sizeof(uint32_t), cudaMemcpyDeviceToDevice,
                                     g->stream));
 
-    fill_plan(a, *dp);
+    fill_plan(g, a, *dp);
     a.x_in = xin;
     a.mm_prev_min = k > 0 ? mm_min + (size_t)(k - 1) * g->G * cf.stride : nullptr;
     a.mm_prev_max = k > 0 ? mm_max + (size_t)(k - 1) * g->G * cf.stride : nullptr;
