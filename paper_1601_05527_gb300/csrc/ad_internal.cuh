@@ -118,6 +118,14 @@ template <> struct Store<float> {
     }
     // value as stored (identity for FP32)
     __device__ __forceinline__ static float round(float f) { return f; }
+    // minimum and maximum of two words of a chunk, value by value, and the words that no value exceeds
+    static constexpr uint32_t kMinInit = 0x7f800000u, kMaxInit = 0xff800000u;
+    __device__ __forceinline__ static uint32_t min_word(uint32_t a, uint32_t b) {
+        return __float_as_uint(fminf(__uint_as_float(a), __uint_as_float(b)));
+    }
+    __device__ __forceinline__ static uint32_t max_word(uint32_t a, uint32_t b) {
+        return __float_as_uint(fmaxf(__uint_as_float(a), __uint_as_float(b)));
+    }
 };
 template <> struct Store<__nv_bfloat16> {
     static constexpr int V = 8;
@@ -138,6 +146,15 @@ template <> struct Store<__nv_bfloat16> {
     }
     __device__ __forceinline__ static float round(float f) {
         return __bfloat162float(__float2bfloat16_rn(f));
+    }
+    static constexpr uint32_t kMinInit = 0x7f807f80u, kMaxInit = 0xff80ff80u;
+    __device__ __forceinline__ static uint32_t min_word(uint32_t a, uint32_t b) {
+        const __nv_bfloat162 h = __hmin2(*reinterpret_cast<__nv_bfloat162 *>(&a), *reinterpret_cast<__nv_bfloat162 *>(&b));
+        return *reinterpret_cast<const uint32_t *>(&h);
+    }
+    __device__ __forceinline__ static uint32_t max_word(uint32_t a, uint32_t b) {
+        const __nv_bfloat162 h = __hmax2(*reinterpret_cast<__nv_bfloat162 *>(&a), *reinterpret_cast<__nv_bfloat162 *>(&b));
+        return *reinterpret_cast<const uint32_t *>(&h);
     }
 };
 
@@ -160,6 +177,15 @@ template <> struct Store<__half> {
         return make_uint4(pack2(f[0], f[1]), pack2(f[2], f[3]), pack2(f[4], f[5]), pack2(f[6], f[7]));
     }
     __device__ __forceinline__ static float round(float f) { return __half2float(__float2half_rn(f)); }
+    static constexpr uint32_t kMinInit = 0x7c007c00u, kMaxInit = 0xfc00fc00u;
+    __device__ __forceinline__ static uint32_t min_word(uint32_t a, uint32_t b) {
+        const __half2 h = __hmin2(*reinterpret_cast<__half2 *>(&a), *reinterpret_cast<__half2 *>(&b));
+        return *reinterpret_cast<const uint32_t *>(&h);
+    }
+    __device__ __forceinline__ static uint32_t max_word(uint32_t a, uint32_t b) {
+        const __half2 h = __hmax2(*reinterpret_cast<__half2 *>(&a), *reinterpret_cast<__half2 *>(&b));
+        return *reinterpret_cast<const uint32_t *>(&h);
+    }
 };
 
 // 16-bit fixed point: q in [-32768, 32767] stands for q * 2^-15 (covers [-1, 1);
@@ -189,6 +215,9 @@ template <> struct Store<Q16> {
         return make_uint4(pack2(f[0], f[1]), pack2(f[2], f[3]), pack2(f[4], f[5]), pack2(f[6], f[7]));
     }
     __device__ __forceinline__ static float round(float f) { return (float)code(f) * kStep; }
+    static constexpr uint32_t kMinInit = 0x7fff7fffu, kMaxInit = 0x80008000u;
+    __device__ __forceinline__ static uint32_t min_word(uint32_t a, uint32_t b) { return __vmins2(a, b); }
+    __device__ __forceinline__ static uint32_t max_word(uint32_t a, uint32_t b) { return __vmaxs2(a, b); }
 };
 
 // ----------------------------------------------------------------------------

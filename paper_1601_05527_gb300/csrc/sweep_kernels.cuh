@@ -412,14 +412,101 @@ __device__ __forceinline__ void smem_max(float *p, float f) {
     else atomicMin(reinterpret_cast<unsigned int *>(p), __float_as_uint(f));
 }
 
-// The min/max of the stored values of one graph, in shared memory: mm[0 ..
-// stride) the minima, then the maxima.  A CTA (batches: a warp) shares one copy;
-// a row that stays inside the bounds met so far -- nearly every row -- only
-// reads them (one wavefront for all rows of a warp), and no lane keeps them in
-// registers, which the gathers need.  mm NULL: straight to the global slots.
-template <typename T, int LPR, int CPL, bool P>
+// The min/max of the stored values of one graph that a warp has met.
+//
+// Single graphs: one copy per CTA in shared memory, mm[0 .. stride) the minima,
+// then the maxima.  A CTA sees thousands of rows; one that stays inside the bounds
+// met so far -- nearly every row -- only reads them (one wavefront for all rows of
+// a warp), and no lane keeps them in registers, which the gathers need.
+template <typename T>
+struct SharedExtremes {
+    static constexpr int V = Store<T>::V;
+    float *mm;
+
+    // the values o of chunk number q of a row (chunk slot c of the lane), stored as v
+    __device__ __forceinline__ void add(const SweepArgs &a, int c, int q, const float (&o)[V], const uint4 &v) {
+#pragma unroll
+        for (int e4 = 0; e4 < V / 4; ++e4) {
+            const float4 lo = ldac(mm + q * V + 4 * e4), hi = ldac(mm + a.stride + q * V + 4 * e4);
+            const float *oo = o + 4 * e4;
+            if (oo[0] < lo.x || oo[1] < lo.y || oo[2] < lo.z || oo[3] < lo.w || oo[0] > hi.x || oo[1] > hi.y ||
+                oo[2] > hi.z || oo[3] > hi.w) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    smem_min(mm + q * V + 4 * e4 + j, oo[j]);
+                    smem_max(mm + a.stride + q * V + 4 * e4 + j, oo[j]);
+                }
+            }
+        }
+    }
+};
+
+// Batches: in registers, as the lane's 16-byte chunks are stored (two values to a
+// word for the 16-bit formats: eight registers a chunk), merged over the lane groups
+// when the warp moves to another graph.  A warp meets a graph for a few tasks only,
+// in which most rows set new bounds: with a copy per warp in shared memory the
+// conflicting atomics took 43% of the L1 pipe (64 Watts-Strogatz graphs of 2,000 to
+// 20,000 vertices, BF16, R = 16: 78 -> 58 us a sweep in registers; 1,000 graphs of
+// 1,000 vertices: 112 -> 77 us, FP32 122 -> 108 us).
+template <typename T, int LPR, int CPL>
+struct RegisterExtremes {
+    using S = Store<T>;
+    static constexpr int V = S::V;
+    uint4 mn[CPL], mx[CPL];
+
+    __device__ __forceinline__ static uint4 min4(const uint4 &x, const uint4 &y) {
+        return make_uint4(S::min_word(x.x, y.x), S::min_word(x.y, y.y), S::min_word(x.z, y.z), S::min_word(x.w, y.w));
+    }
+    __device__ __forceinline__ static uint4 max4(const uint4 &x, const uint4 &y) {
+        return make_uint4(S::max_word(x.x, y.x), S::max_word(x.y, y.y), S::max_word(x.z, y.z), S::max_word(x.w, y.w));
+    }
+    __device__ __forceinline__ static uint4 shfl_xor4(const uint4 &x, int o) {
+        return make_uint4(__shfl_xor_sync(0xffffffffu, x.x, o), __shfl_xor_sync(0xffffffffu, x.y, o),
+                          __shfl_xor_sync(0xffffffffu, x.z, o), __shfl_xor_sync(0xffffffffu, x.w, o));
+    }
+    __device__ __forceinline__ void reset() {
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) {
+            mn[c] = make_uint4(S::kMinInit, S::kMinInit, S::kMinInit, S::kMinInit);
+            mx[c] = make_uint4(S::kMaxInit, S::kMaxInit, S::kMaxInit, S::kMaxInit);
+        }
+    }
+    __device__ __forceinline__ void add(const SweepArgs &a, int c, int q, const float (&o)[V], const uint4 &v) {
+        mn[c] = min4(mn[c], v);
+        mx[c] = max4(mx[c], v);
+    }
+    // merge into the global slots of graph g; all 32 lanes
+    __device__ __forceinline__ void flush(const SweepArgs &a, int g, int lane) {
+#pragma unroll
+        for (int o = LPR; o < 32; o <<= 1)
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) {
+                mn[c] = min4(mn[c], shfl_xor4(mn[c], o));
+                mx[c] = max4(mx[c], shfl_xor4(mx[c], o));
+            }
+        uint32_t *gmin = a.mm_min + (size_t)g * a.stride, *gmax = a.mm_max + (size_t)g * a.stride;
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) {
+            const int q = lane + c * LPR;
+            if (lane < LPR && q < a.nchunks) {
+                float lo[V], hi[V];
+                S::unpack(mn[c], lo);
+                S::unpack(mx[c], hi);
+#pragma unroll
+                for (int e = 0; e < V; ++e)
+                    if (lo[e] <= hi[e]) {   // (no row: not so)
+                        atomicMin(gmin + q * V + e, f2ord(lo[e]));
+                        atomicMax(gmax + q * V + e, f2ord(hi[e]));
+                    }
+            }
+        }
+    }
+};
+
+// in: the row is of the graph that x describes; otherwise its values go to the global slots
+template <typename T, int LPR, int CPL, bool P, typename X>
 __device__ __forceinline__ void row_epilogue(const SweepArgs &a, int64_t row, int gl, const uint4 (&own)[CPL],
-                                             const float (&S)[CPL * Store<T>::V], const float *acg, float *mm,
+                                             const float (&S)[CPL * Store<T>::V], const float *acg, X &x, bool in,
                                              uint32_t *gmin, uint32_t *gmax) {
     constexpr int V = Store<T>::V;
     uint4 *Y = reinterpret_cast<uint4 *>(a.x_out);
@@ -444,21 +531,10 @@ __device__ __forceinline__ void row_epilogue(const SweepArgs &a, int64_t row, in
                     o[e] = Store<T>::round(A[j] * (z - C[j]));
                 }
             }
-            Y[row * row_q + q] = Store<T>::pack(o);
-            if (mm) {
-#pragma unroll
-                for (int e4 = 0; e4 < V / 4; ++e4) {
-                    const float4 lo = ldac(mm + q * V + 4 * e4), hi = ldac(mm + a.stride + q * V + 4 * e4);
-                    const float *oo = o + 4 * e4;
-                    if (oo[0] < lo.x || oo[1] < lo.y || oo[2] < lo.z || oo[3] < lo.w || oo[0] > hi.x || oo[1] > hi.y ||
-                        oo[2] > hi.z || oo[3] > hi.w) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            smem_min(mm + q * V + 4 * e4 + j, oo[j]);
-                            smem_max(mm + a.stride + q * V + 4 * e4 + j, oo[j]);
-                        }
-                    }
-                }
+            const uint4 v = Store<T>::pack(o);
+            Y[row * row_q + q] = v;
+            if (in) {
+                x.add(a, c, q, o, v);
             } else {
 #pragma unroll
                 for (int e = 0; e < V; ++e) {
@@ -528,42 +604,29 @@ __global__ void k_scale_center(const uint32_t *pmin, const uint32_t *pmax, const
 }
 
 // ----------------------------------------------------------------------------
-// The graph a warp of a batch is in: its vertex range and min/max copy, flushed
-// to the global slots when the warp moves to another graph (tasks are ordered by
+// The graph a warp of a batch is in: its vertex range and min/max, which go to
+// the global slots when the warp moves to another graph (tasks are ordered by
 // vertex, so a warp meets few).  A row of yet another graph in the same warp (at
 // the border of two graphs) goes to the global slots directly.
 // ----------------------------------------------------------------------------
-template <typename T>
+template <typename T, int LPR, int CPL>
 struct WarpGraph {
     int g = -1;
     int32_t lo = 0, hi = 0;   // vertices of graph g
+    RegisterExtremes<T, LPR, CPL> x;
 
-    __device__ __forceinline__ void reset(const SweepArgs &a, float *mm, int lane) {
-        for (int r = lane; r < a.stride; r += 32) {
-            mm[r] = INFINITY;
-            mm[a.stride + r] = -INFINITY;
-        }
-        __syncwarp();
-    }
-    __device__ __forceinline__ void flush(const SweepArgs &a, const float *mm, int lane) const {
-        __syncwarp();
-        if (g < 0) return;
-        for (int r = lane; r < a.nchunks * Store<T>::V; r += 32)
-            if (mm[r] <= mm[a.stride + r]) {
-                atomicMin(a.mm_min + (size_t)g * a.stride + r, f2ord(mm[r]));
-                atomicMax(a.mm_max + (size_t)g * a.stride + r, f2ord(mm[a.stride + r]));
-            }
-        __syncwarp();
+    __device__ __forceinline__ void flush(const SweepArgs &a, int lane) {
+        if (g >= 0) x.flush(a, g, lane);
     }
     // all 32 lanes; have: the lane has a row.  True: the row is in graph g.
-    __device__ __forceinline__ bool enter(const SweepArgs &a, float *mm, int lane, bool have, int32_t row) {
+    __device__ __forceinline__ bool enter(const SweepArgs &a, int lane, bool have, int32_t row) {
         if (__any_sync(0xffffffffu, have && !(row >= lo && row < hi))) {
-            flush(a, mm, lane);
+            flush(a, lane);
             const int last = __reduce_max_sync(0xffffffffu, have ? row : -1);
             g = graph_of(a.voff, a.G, last);
             lo = (int32_t)__ldg(a.voff + g);
             hi = (int32_t)__ldg(a.voff + g + 1);
-            reset(a, mm, lane);
+            x.reset();
         }
         return row >= lo && row < hi;
     }
@@ -615,7 +678,7 @@ constexpr int sweep_loads() { return sizeof(T) == 4 ? AD_SWEEP_UB : AD_SWEEP_UB1
 // The tasks of one sweep on this CTA, then the CTA's min/max to the sweep's
 // slots.  P: inside the persistent launch.  B: a batch of graphs.  acs: scale and
 // centre of a single graph in shared memory (batches read them from a.ac); mm:
-// its min/max copy, initialised (batches: one per warp).
+// its min/max copy, initialised (batches have none).
 template <typename T, int LPR, int CPL, bool P, bool B>
 __device__ __forceinline__ void sweep_tasks(const SweepArgs &a, const float *acs, float *mm) {
     using L = Lane<T, LPR, CPL>;
@@ -625,22 +688,20 @@ __device__ __forceinline__ void sweep_tasks(const SweepArgs &a, const float *acs
     const int lane = threadIdx.x & 31;
     const int grp = lane / LPR, gl = lane % LPR;
 
-    WarpGraph<T> wg;
-    if (B) {
-        mm += (threadIdx.x >> 5) * 2 * a.stride;
-        wg.reset(a, mm, lane);
-    }
+    WarpGraph<T, LPR, CPL> wg;   // batches
+    if (B) wg.x.reset();
+    SharedExtremes<T> cta{mm};   // single graphs
     // epilogue of the lanes with a row (writer: the lane stores a part of it)
     auto finish = [&](int32_t row, bool have, bool writer, const uint4 (&own)[CPL], const float (&S)[E]) {
         if (B) {
-            const bool in = wg.enter(a, mm, lane, have, row);
+            const bool in = wg.enter(a, lane, have, row);
             if (writer) {
                 const int g = in ? wg.g : graph_of(a.voff, a.G, row);
-                row_epilogue<T, LPR, CPL, P>(a, row, gl, own, S, a.ac + (size_t)g * 2 * a.stride, in ? mm : nullptr,
+                row_epilogue<T, LPR, CPL, P>(a, row, gl, own, S, a.ac + (size_t)g * 2 * a.stride, wg.x, in,
                                              a.mm_min + (size_t)g * a.stride, a.mm_max + (size_t)g * a.stride);
             }
         } else if (writer) {
-            row_epilogue<T, LPR, CPL, P>(a, row, gl, own, S, acs, mm, nullptr, nullptr);
+            row_epilogue<T, LPR, CPL, P>(a, row, gl, own, S, acs, cta, true, nullptr, nullptr);
         }
     };
 
@@ -720,7 +781,7 @@ __device__ __forceinline__ void sweep_tasks(const SweepArgs &a, const float *acs
         }
     }
     if (B) {
-        wg.flush(a, mm, lane);
+        wg.flush(a, lane);
         return;
     }
     __syncthreads();
@@ -731,10 +792,10 @@ __device__ __forceinline__ void sweep_tasks(const SweepArgs &a, const float *acs
         }
 }
 
-// Shared memory of a sweep: [2][stride] scale and centre, then the min/max
-// copies, [2][stride] each (one for a single graph, one per warp for a batch).
+// Shared memory of a sweep of a single graph: [2][stride] scale and centre, then
+// [2][stride] min/max.  Batches use none.
 __host__ __device__ constexpr size_t sweep_smem(int stride, bool batch) {
-    return (size_t)(2 + 2 * (batch ? 8 : 1)) * stride * sizeof(float);
+    return batch ? 0 : (size_t)4 * stride * sizeof(float);
 }
 
 __device__ __forceinline__ void reset_minmax(int32_t stride, float *mm) {
