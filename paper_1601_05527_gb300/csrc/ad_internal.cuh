@@ -403,6 +403,7 @@ ad_status sweep_step(ad_graph_t g, ad_storage storage, int32_t R, double omega, 
                      const uint32_t *pmin, const uint32_t *pmax, uint32_t *mn, uint32_t *mx);
 ad_status get_row_plan(ad_graph_t g, int groups, bool upper, RowPlan **out);
 void natural_shape(int R, ad_storage storage, int *lanes_per_row, int *chunks_per_lane);   // sweep.cu
+ad_status shape_ctas(ad_graph_t g, int R, ad_storage storage, int lanes_per_row, int chunks_per_lane, int *per_sm);
 
 // selection (select.cu)
 ad_status select_whole_graph(ad_graph_t g, const float *score_dev, double fraction, ad_mode mode,

@@ -443,8 +443,12 @@ extern "C" ad_status ad_graph_autotune(ad_graph_t g, int32_t R, ad_storage stora
     std::vector<Cand> cands;
     std::vector<std::pair<int, int>> shapes = {{nat_lpr, nat_cpl}};
     if (nat_lpr >= 2 && nat_cpl == 1) shapes.push_back({nat_lpr / 2, 2});
-    for (const auto &sh : shapes)
-        for (int per_sm : {0, 5, 4}) cands.push_back({sh.first, sh.second, per_sm});
+    for (const auto &sh : shapes) {   // as many CTAs per SM as fit (0), and fewer
+        int fit = 0;
+        AD_TRY(shape_ctas(g, R, storage, sh.first, sh.second, &fit));
+        for (int per_sm : {0, 5, 4})
+            if (per_sm < fit) cands.push_back({sh.first, sh.second, per_sm});
+    }
     int best = 0;
     float best_ms = 0.f;
     if (g->m > 0) {

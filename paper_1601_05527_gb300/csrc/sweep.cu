@@ -40,6 +40,19 @@ void natural_shape(int R, ad_storage storage, int *lpr, int *cpl) {
     *cpl = c.cpl;
 }
 
+ad_status shape_ctas(ad_graph_t g, int R, ad_storage storage, int lpr, int cpl, int *per_sm) {
+    Config c = natural_config(R, storage);
+    c.lpr = lpr;
+    c.cpl = cpl;
+    const bool batch = g->G > 1;
+    switch (storage) {
+        case AD_STORAGE_BF16: return ctas_bf16(c, batch, per_sm);
+        case AD_STORAGE_FP16: return ctas_f16(c, batch, per_sm);
+        case AD_STORAGE_Q16: return ctas_q16(c, batch, per_sm);
+        default: return ctas_f32(c, batch, per_sm);
+    }
+}
+
 static Config pick_config(ad_graph_t g, int R, ad_storage storage) {
     Config c = natural_config(R, storage);
     for (const auto &t : g->tuned)

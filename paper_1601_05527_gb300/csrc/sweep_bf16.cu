@@ -8,6 +8,8 @@ ad_status dispatch_bf16(ad_graph_t g, const Config &cf, bool sweep, const SweepA
     return dispatch<__nv_bfloat16>(g, cf, sweep, a, n_tasks, smem);
 }
 
+ad_status ctas_bf16(const Config &cf, bool batch, int *per_sm) { return sweep_ctas<__nv_bfloat16>(cf, batch, per_sm); }
+
 ad_status relax_bf16(ad_graph_t g, const Config &cf, RelaxArgs &r) { return relax_dispatch<__nv_bfloat16>(g, cf, r); }
 
 ad_status launch_init_bf16(ad_graph_t g, int blocks, int32_t stride, uint64_t seed, uint32_t stream_id, void *x) {

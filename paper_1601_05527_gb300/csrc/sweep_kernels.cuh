@@ -1115,11 +1115,33 @@ int blocks_for(bool sweep, bool batch, size_t smem) {
     return per_sm > 0 ? per_sm : 1;
 }
 
+// f(lanes per row, chunks per lane) for a sweep or distance shape, as constants
+template <typename F>
+ad_status with_shape(const Config &cf, F f) {
+    using std::integral_constant;
+    switch (cf.lpr * 100 + cf.cpl) {
+        case 101: return f(integral_constant<int, 1>{}, integral_constant<int, 1>{});
+        case 201: return f(integral_constant<int, 2>{}, integral_constant<int, 1>{});
+        case 401: return f(integral_constant<int, 4>{}, integral_constant<int, 1>{});
+        case 801: return f(integral_constant<int, 8>{}, integral_constant<int, 1>{});
+        case 1601: return f(integral_constant<int, 16>{}, integral_constant<int, 1>{});
+        case 3201: return f(integral_constant<int, 32>{}, integral_constant<int, 1>{});
+        case 3202: return f(integral_constant<int, 32>{}, integral_constant<int, 2>{});
+        // fewer lanes per row, more chunks per lane: the alternative shapes the autotuner tries
+        case 102: return f(integral_constant<int, 1>{}, integral_constant<int, 2>{});
+        case 202: return f(integral_constant<int, 2>{}, integral_constant<int, 2>{});
+        case 402: return f(integral_constant<int, 4>{}, integral_constant<int, 2>{});
+        case 802: return f(integral_constant<int, 8>{}, integral_constant<int, 2>{});
+        case 1602: return f(integral_constant<int, 16>{}, integral_constant<int, 2>{});
+        default: return fail(AD_ERR_INVALID_ARG, "unsupported R / storage combination");
+    }
+}
+
 template <typename T>
 ad_status dispatch(ad_graph_t g, const Config &cf, bool sweep, const SweepArgs &a, int64_t n_tasks,
                           size_t smem) {
     // persistent grid: every SM full, but no more warps than tasks
-    auto run = [&](auto lpr_c, auto cpl_c) -> ad_status {
+    return with_shape(cf, [&](auto lpr_c, auto cpl_c) -> ad_status {
         constexpr int LPR = decltype(lpr_c)::value, CPL = decltype(cpl_c)::value;
         int per_sm = blocks_for<T, LPR, CPL>(sweep, a.G > 1, smem);
         if (sweep && cf.per_sm > 0 && cf.per_sm < per_sm) per_sm = cf.per_sm;
@@ -1128,26 +1150,17 @@ ad_status dispatch(ad_graph_t g, const Config &cf, bool sweep, const SweepArgs &
         if (blocks > need) blocks = need > 0 ? need : 1;
         return sweep ? launch_sweep<T, LPR, CPL>(g, a, (int)blocks, smem)
                      : launch_distance<T, LPR, CPL>(g, a, (int)blocks);
-    };
-    using std::integral_constant;
-    switch (cf.lpr * 100 + cf.cpl) {
-        case 101: return run(integral_constant<int, 1>{}, integral_constant<int, 1>{});
-        case 201: return run(integral_constant<int, 2>{}, integral_constant<int, 1>{});
-        case 401: return run(integral_constant<int, 4>{}, integral_constant<int, 1>{});
-        case 801: return run(integral_constant<int, 8>{}, integral_constant<int, 1>{});
-        case 1601: return run(integral_constant<int, 16>{}, integral_constant<int, 1>{});
-        case 3201: return run(integral_constant<int, 32>{}, integral_constant<int, 1>{});
-        case 3202: return run(integral_constant<int, 32>{}, integral_constant<int, 2>{});
-        // fewer lanes per row, more chunks per lane: the alternative shapes the autotuner tries
-        case 102: return run(integral_constant<int, 1>{}, integral_constant<int, 2>{});
-        case 202: return run(integral_constant<int, 2>{}, integral_constant<int, 2>{});
-        case 402: return run(integral_constant<int, 4>{}, integral_constant<int, 2>{});
-        case 802: return run(integral_constant<int, 8>{}, integral_constant<int, 2>{});
-        case 1602: return run(integral_constant<int, 16>{}, integral_constant<int, 2>{});
-        default: return fail(AD_ERR_INVALID_ARG, "unsupported R / storage combination");
-    }
+    });
 }
 
+// CTAs of the sweep that fit on an SM
+template <typename T>
+ad_status sweep_ctas(const Config &cf, bool batch, int *per_sm) {
+    return with_shape(cf, [&](auto lpr_c, auto cpl_c) -> ad_status {
+        *per_sm = blocks_for<T, decltype(lpr_c)::value, decltype(cpl_c)::value>(true, batch, sweep_smem(cf.stride, batch));
+        return AD_OK;
+    });
+}
 
 // Persistent launch of k_relax: every CTA co-resident (cooperative launch),
 // as many as fit or as the larger of the two plans can use.
@@ -1191,6 +1204,10 @@ ad_status dispatch_f32(ad_graph_t g, const Config &cf, bool sweep, const SweepAr
 ad_status dispatch_bf16(ad_graph_t g, const Config &cf, bool sweep, const SweepArgs &a, int64_t n_tasks, size_t smem);
 ad_status dispatch_f16(ad_graph_t g, const Config &cf, bool sweep, const SweepArgs &a, int64_t n_tasks, size_t smem);
 ad_status dispatch_q16(ad_graph_t g, const Config &cf, bool sweep, const SweepArgs &a, int64_t n_tasks, size_t smem);
+ad_status ctas_f32(const Config &cf, bool batch, int *per_sm);
+ad_status ctas_bf16(const Config &cf, bool batch, int *per_sm);
+ad_status ctas_f16(const Config &cf, bool batch, int *per_sm);
+ad_status ctas_q16(const Config &cf, bool batch, int *per_sm);
 ad_status relax_f32(ad_graph_t g, const Config &cf, RelaxArgs &r);
 ad_status relax_bf16(ad_graph_t g, const Config &cf, RelaxArgs &r);
 ad_status relax_f16(ad_graph_t g, const Config &cf, RelaxArgs &r);

@@ -8,6 +8,8 @@ ad_status dispatch_q16(ad_graph_t g, const Config &cf, bool sweep, const SweepAr
     return dispatch<Q16>(g, cf, sweep, a, n_tasks, smem);
 }
 
+ad_status ctas_q16(const Config &cf, bool batch, int *per_sm) { return sweep_ctas<Q16>(cf, batch, per_sm); }
+
 ad_status relax_q16(ad_graph_t g, const Config &cf, RelaxArgs &r) { return relax_dispatch<Q16>(g, cf, r); }
 
 ad_status launch_init_q16(ad_graph_t g, int blocks, int32_t stride, uint64_t seed, uint32_t stream_id, void *x) {
