@@ -553,7 +553,9 @@ static ad_status count_kept(ad_graph_t g, const uint8_t *keep, int64_t m, int64_
 }
 
 // Finest edges behind every edge of a coarse level: mult of level l + 1 from mult
-// of level l (NULL at level 0: one each).
+// of level l (NULL at level 0: one each).  32 bits hold them: the structures of a
+// level of 2^32 edges (48 bytes an edge, 24 more while it is coarsened) exceed the
+// device's memory.
 __global__ void k_mult_up(const int64_t *f2c, const uint32_t *mult_f, int64_t m, uint32_t *mult_c) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e < m && f2c[e] >= 0) atomicAdd(mult_c + f2c[e], mult_f ? mult_f[e] : 1u);

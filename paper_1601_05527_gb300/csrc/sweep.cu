@@ -136,7 +136,7 @@ ad_status sweep_step(ad_graph_t g, ad_storage storage, int32_t R, double omega, 
     a.omega = (float)omega;
     a.voff = g->voff; a.G = g->G; a.blocked = g->G > 1 ? 1 : 0;
     a.anchor = g->anchor;
-    AD_TRY(ensure(g, g->ac, (size_t)g->G * 2 * cf.stride * sizeof(float)));
+    if (g->G > 1) AD_TRY(ensure(g, g->ac, (size_t)g->G * 2 * cf.stride * sizeof(float)));   // single graphs: shared memory
     a.ac = static_cast<float *>(g->ac.ptr);
     fill_plan(g, a, *sp);
     a.x_in = x_in; a.x_out = x_out;
@@ -295,7 +295,7 @@ ad_status algebraic_distance(ad_graph_t g, int32_t R, int32_t k, double omega, u
     a.G = g->G;
     a.blocked = g->G > 1 ? 1 : 0;
     a.anchor = g->anchor;
-    AD_TRY(ensure(g, g->ac, (size_t)g->G * 2 * cf.stride * sizeof(float)));
+    if (g->G > 1) AD_TRY(ensure(g, g->ac, (size_t)g->G * 2 * cf.stride * sizeof(float)));   // single graphs: shared memory
     a.ac = static_cast<float *>(g->ac.ptr);
 
     void *xin = g->x0.ptr, *xout = g->x1.ptr;
