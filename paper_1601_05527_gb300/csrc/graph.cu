@@ -236,61 +236,18 @@ __global__ void k_degrees(const int64_t *rp, const int32_t *col, const float *w,
 // lane.  exact_out[i] records which case row i is (the seed rule relies on it).
 __device__ __forceinline__ int fp32_biased_exponent(float v) { return (int)((__float_as_uint(v) >> 23) & 0xffu); }
 
-// Rows longer than kLongDegreeRow are left out: one warp would hold the launch up on
-// a hub for milliseconds (R-MAT 22: 4.9 ms, all of it hubs); k_wdegrees_long gives
-// each a block.
+// Rows longer than kLongDegreeRow take a block each, the first `long_blocks` of the
+// launch: one warp would hold it up on a hub for milliseconds (R-MAT 22: 4.9 ms, all
+// of it hubs), and a launch of their own after the others costs its latency and drain
+// (a weight update of R-MAT 14 146 -> 133 us, R-MAT 16 208 -> 191 us, R-MAT 22 14.6 ->
+// 12.9 ms in one launch).
 constexpr int64_t kLongDegreeRow = 2048;
+constexpr int kDegreeThreads = 512;
 __device__ __forceinline__ bool sum_is_exact(int64_t d, int emax, int emin) {
     int lg = 0;
     while (((int64_t)1 << lg) < d) ++lg;   // ceil(log2 d)
     // bits spanned by every partial sum: (emax - 127 + 1 + lg) - (max(emin, 1) - 150)
     return d == 0 || emax - max(emin, 1) + lg + 24 <= 53;
-}
-
-__global__ void k_wdegrees(const int64_t *rp, const float *w, int64_t n, double *D, float *Dinv, uint8_t *exact_out) {
-    const int lane = threadIdx.x & 31;
-    const int64_t W = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t i = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += W) {
-        const int64_t b = rp[i], e = rp[i + 1];
-        if (e - b > kLongDegreeRow) continue;
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;   // four independent loads in flight per lane
-        int emax = 0, emin = 255;
-        int64_t p = b + lane;
-        for (; p + 96 < e; p += 128) {
-            const float w0 = w[p], w1 = w[p + 32], w2 = w[p + 64], w3 = w[p + 96];
-            s0 += (double)w0;
-            s1 += (double)w1;
-            s2 += (double)w2;
-            s3 += (double)w3;
-            emax = max(emax, max(max(fp32_biased_exponent(w0), fp32_biased_exponent(w1)),
-                                 max(fp32_biased_exponent(w2), fp32_biased_exponent(w3))));
-            emin = min(emin, min(min(fp32_biased_exponent(w0), fp32_biased_exponent(w1)),
-                                 min(fp32_biased_exponent(w2), fp32_biased_exponent(w3))));
-        }
-        for (; p < e; p += 32) {
-            const float w0 = w[p];
-            s0 += (double)w0;
-            emax = max(emax, fp32_biased_exponent(w0));
-            emin = min(emin, fp32_biased_exponent(w0));
-        }
-        double s = (s0 + s1) + (s2 + s3);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            s += __shfl_xor_sync(0xffffffffu, s, o);
-            emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
-            emin = min(emin, __shfl_xor_sync(0xffffffffu, emin, o));
-        }
-        const bool exact = sum_is_exact(e - b, emax, emin);
-        if (lane == 0) {
-            if (!exact) {   // the plain definition's order, one entry after the other
-                s = 0.0;
-                for (int64_t q = b; q < e; ++q) s += (double)w[q];
-            }
-            D[i] = s;
-            Dinv[i] = s > 0.0 ? (float)(1.0 / s) : 0.f;
-            exact_out[i] = exact ? 1 : 0;
-        }
-    }
 }
 
 // The rows of more than kLongDegreeRow entries, in any order: they do not change with
@@ -300,18 +257,16 @@ __global__ void k_list_long_rows(const int64_t *rp, int64_t n, int32_t *rows, un
         if (rp[i + 1] - rp[i] > kLongDegreeRow) rows[atomicAdd(count, 1u)] = (int32_t)i;
 }
 
-// The long rows, a block each: the same sum where it is exact, otherwise
-// one after the other in CSR order by one thread, from shared memory.
-constexpr int kLongDegreeThreads = 512;
-__global__ void __launch_bounds__(kLongDegreeThreads) k_wdegrees_long(const int64_t *rp, const float *w,
-                                                                      const int32_t *rows, int64_t count, double *D,
-                                                                      float *Dinv, uint8_t *exact_out) {
-    constexpr int T = kLongDegreeThreads, NW = T / 32, kTile = 4 * T;
+// The long rows, a block each: the same sum where it is exact in any order,
+// otherwise one after the other in CSR order by one thread, from shared memory.
+__device__ __forceinline__ void long_degrees(const int64_t *rp, const float *w, const int32_t *rows, int64_t count,
+                                             int blocks, double *D, float *Dinv, uint8_t *exact_out) {
+    constexpr int T = kDegreeThreads, NW = T / 32, kTile = 4 * T;
     __shared__ double ssum[NW];
     __shared__ int smax[NW], smin[NW];
     __shared__ float tile[kTile];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t t = blockIdx.x; t < count; t += gridDim.x) {
+    for (int64_t t = blockIdx.x; t < count; t += blocks) {
         const int64_t i = rows[t], b = rp[i], e = rp[i + 1];
         double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
         int emax = 0, emin = 255;
@@ -375,6 +330,58 @@ __global__ void __launch_bounds__(kLongDegreeThreads) k_wdegrees_long(const int6
             exact_out[i] = exact ? 1 : 0;
         }
         __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kDegreeThreads) k_wdegrees(const int64_t *rp, const float *w, int64_t n,
+                                                             const int32_t *rows, int64_t n_rows, int long_blocks,
+                                                             double *D, float *Dinv, uint8_t *exact_out) {
+    if (blockIdx.x < long_blocks) {
+        long_degrees(rp, w, rows, n_rows, long_blocks, D, Dinv, exact_out);
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    const int64_t W = (int64_t)(gridDim.x - long_blocks) * (blockDim.x >> 5);
+    for (int64_t i = (blockIdx.x - long_blocks) * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += W) {
+        const int64_t b = rp[i], e = rp[i + 1];
+        if (e - b > kLongDegreeRow) continue;
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;   // four independent loads in flight per lane
+        int emax = 0, emin = 255;
+        int64_t p = b + lane;
+        for (; p + 96 < e; p += 128) {
+            const float w0 = w[p], w1 = w[p + 32], w2 = w[p + 64], w3 = w[p + 96];
+            s0 += (double)w0;
+            s1 += (double)w1;
+            s2 += (double)w2;
+            s3 += (double)w3;
+            emax = max(emax, max(max(fp32_biased_exponent(w0), fp32_biased_exponent(w1)),
+                                 max(fp32_biased_exponent(w2), fp32_biased_exponent(w3))));
+            emin = min(emin, min(min(fp32_biased_exponent(w0), fp32_biased_exponent(w1)),
+                                 min(fp32_biased_exponent(w2), fp32_biased_exponent(w3))));
+        }
+        for (; p < e; p += 32) {
+            const float w0 = w[p];
+            s0 += (double)w0;
+            emax = max(emax, fp32_biased_exponent(w0));
+            emin = min(emin, fp32_biased_exponent(w0));
+        }
+        double s = (s0 + s1) + (s2 + s3);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+            emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+            emin = min(emin, __shfl_xor_sync(0xffffffffu, emin, o));
+        }
+        const bool exact = sum_is_exact(e - b, emax, emin);
+        if (lane == 0) {
+            if (!exact) {   // the plain definition's order, one entry after the other
+                s = 0.0;
+                for (int64_t q = b; q < e; ++q) s += (double)w[q];
+            }
+            D[i] = s;
+            Dinv[i] = s > 0.0 ? (float)(1.0 / s) : 0.f;
+            exact_out[i] = exact ? 1 : 0;
+        }
     }
 }
 
@@ -476,19 +483,18 @@ ad_status recompute_degrees(ad_graph_t g) {
     AD_LAUNCH(k_degrees, (int)tblocks, 256, 0, g->stream, g->rp, g->col, g->w, g->n, g->D, g->Dinv, g->upos,
               ucount);
     if (g->w) {
-        const int64_t wblocks = std::min<int64_t>((g->n + 7) / 8 + 1, (int64_t)g->num_sms * 64);
+        constexpr int kRows = kDegreeThreads / 32;   // rows of a block, a warp each
+        const int64_t wblocks = std::min<int64_t>((g->n + kRows - 1) / kRows + 1, (int64_t)g->num_sms * 32);
         if (!g->dexact) AD_TRY(dalloc_t(g, g->n + 1, &g->dexact));
-        AD_LAUNCH(k_wdegrees, (int)wblocks, 256, 0, g->stream, g->rp, g->w, g->n, g->D, g->Dinv, g->dexact);
-        if (g->n_long_rows > 0) {
-            if (!g->long_rows) {   // the last slot counts while the list is filled
-                AD_TRY(dalloc_t(g, g->n_long_rows + 1, &g->long_rows));
-                unsigned int *count = reinterpret_cast<unsigned int *>(g->long_rows + g->n_long_rows);
-                AD_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(unsigned int), g->stream));
-                AD_LAUNCH(k_list_long_rows, (int)tblocks, 256, 0, g->stream, g->rp, g->n, g->long_rows, count);
-            }
-            AD_LAUNCH(k_wdegrees_long, (int)std::min<int64_t>(g->n_long_rows, (int64_t)g->num_sms * 4), kLongDegreeThreads,
-                      0, g->stream, g->rp, g->w, g->long_rows, g->n_long_rows, g->D, g->Dinv, g->dexact);
+        if (g->n_long_rows > 0 && !g->long_rows) {   // the last slot counts while the list is filled
+            AD_TRY(dalloc_t(g, g->n_long_rows + 1, &g->long_rows));
+            unsigned int *count = reinterpret_cast<unsigned int *>(g->long_rows + g->n_long_rows);
+            AD_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(unsigned int), g->stream));
+            AD_LAUNCH(k_list_long_rows, (int)tblocks, 256, 0, g->stream, g->rp, g->n, g->long_rows, count);
         }
+        const int lblocks = (int)std::min<int64_t>(g->n_long_rows, (int64_t)g->num_sms * 4);
+        AD_LAUNCH(k_wdegrees, (int)wblocks + lblocks, kDegreeThreads, 0, g->stream, g->rp, g->w, g->n, g->long_rows,
+                  g->n_long_rows, lblocks, g->D, g->Dinv, g->dexact);
     }
     int64_t m = 0;
     ad_status st = exclusive_scan_i64(g, ucount, g->eoff, g->n, &m);
